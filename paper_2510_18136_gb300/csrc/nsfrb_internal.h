@@ -16,6 +16,7 @@ constexpr int kMaxSub = 32;               // subbands per plan
 constexpr int kMaxT = 4096;               // longest window
 constexpr int kMaxTRegs = 1247;           // longest window of the register path (32 lanes x 39 samples - 1)
 constexpr int kLongC = 128;               // "chunk" of longer windows: the long-window kernel
+constexpr int kShortT = 64;               // longest window of the short-window kernel
 constexpr int kSmallMax = 16;             // widths <= min(C, 16) use the in-lane path
 constexpr int kHistBins = 256;            // radix-select digit bins (MAD mode)
 
@@ -96,6 +97,7 @@ struct SearchParams {
                            // pixel with its own buffers; long-window kernel: warps per CTA
     int32_t nb;            // barrier-free kernel: pixel buffers per team, 2 (the pixel after next
                            // copied while one is searched) or 1 (the next copied after a pixel)
+    int32_t short_w;       // > 0: the short-window kernel with this many warps per CTA
     // ---- outputs (indexed by absolute pixel)
     PixRec *rec;
     float *full_snr;       // [pix][n_dm][n_w] or nullptr
@@ -169,6 +171,11 @@ int long_warps(const SearchParams &p, int max_smem);
 size_t long_smem(const SearchParams &p, int n_warps);
 cudaError_t launch_search_long(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t prepare_search_long(size_t smem);
+// The short-window kernel: warps per CTA where it applies (0: it does not), and its shared memory.
+int short_warps(const SearchParams &p, int max_smem);
+size_t short_smem(const SearchParams &p, int n_warps);
+cudaError_t launch_search_short(const SearchParams &p, size_t smem, cudaStream_t s);
+cudaError_t prepare_search_short(size_t smem);
 
 // Compaction of per-pixel records into the candidate list ordered by pixel.
 cudaError_t launch_compact(const PixRec *rec, int64_t n_pix, int32_t nx, float thr,

@@ -36,6 +36,7 @@ nsfrb_status cuda_check(nsfrb_plan_s *p, cudaError_t e, const char *what) {
 }
 
 cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, cudaStream_t s) {
+    if (p.short_w > 0) return launch_search_short(p, smem, s);
     switch (C) {
         case 1: return launch_search_c1(p, grid, smem, s);
         case 3: return launch_search_c3(p, grid, smem, s);
@@ -51,6 +52,10 @@ cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, c
 }
 
 cudaError_t prepare_search(int C, size_t smem) {
+    if (C <= 3) {   // windows the short-window kernel may take
+        const cudaError_t e = prepare_search_short(smem);
+        if (e != cudaSuccess) return e;
+    }
     switch (C) {
         case 1: return prepare_search_c1(smem);
         case 3: return prepare_search_c3(smem);
@@ -126,6 +131,15 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
         if (w < 1) return false;
         sp.teams = w;
         smem = long_smem(sp, w);
+        return true;
+    }
+    // windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel
+    // is asked for: a lane per pixel instead of a warp per DM row (SHORT_RULE)
+    if (const int w = tile_pref == 0 ? short_warps(sp, max_smem) : 0) {
+        sp.pipe = 0;
+        sp.stage = 0;
+        sp.short_w = w;
+        smem = short_smem(sp, w);
         return true;
     }
     const uintptr_t base = reinterpret_cast<uintptr_t>(sp.cube);
@@ -204,6 +218,7 @@ bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem) {
 void note_tile(nsfrb_plan_s *pl, const SearchParams &sp) {
     pl->last_tile = sp.pipe ? 10 * sp.teams + sp.nb : 0;
     pl->last_tile_st = sp.dtype;
+    pl->last_short = sp.short_w > 0;
 }
 
 nsfrb_status ensure_device(nsfrb_plan_s *pl) {
@@ -738,14 +753,25 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
     if (st == NSFRB_OK) st = nsfrb_last_timing(plan, nullptr, nullptr);
     if (st != NSFRB_OK) return st;
     const int s_t = plan->last_tile_st;
-    if (plan->last_tile == 0 || s_t < 0) {
+    if ((plan->last_tile == 0 && !plan->last_short) || s_t < 0) {
         if (h_tile) *h_tile = 0;
         return NSFRB_OK;
     }
     const int32_t keep = plan->tile[s_t];
     int32_t best = 0;
     float best_ms = 0.0f;
+    bool timed = false;   // best_ms holds a time
     std::vector<float> t(reps);
+    if (plan->last_short) {   // tile 0 is the short-window kernel: a contender of its own
+        for (int r = 0; r < reps; ++r) {
+            st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
+            if (st == NSFRB_OK) st = nsfrb_last_timing(plan, &t[r], nullptr);
+            if (st != NSFRB_OK) return st;
+        }
+        std::sort(t.begin(), t.end());
+        best_ms = t[reps / 2];
+        timed = true;
+    }
     for (int k = 0; k < NSFRB_N_TILES; ++k) {
         plan->tile[s_t] = kTileCodes[k];
         for (int r = -1; r < reps; ++r) {   // one warm-up search per tile
@@ -761,12 +787,13 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
         std::sort(t.begin(), t.end());
         const float med = t[reps / 2];
         if (h_ms) h_ms[k] = med;
-        if (best == 0 || med < best_ms) {
+        if (!timed || med < best_ms) {
             best = kTileCodes[k];
             best_ms = med;
+            timed = true;
         }
     }
-    plan->tile[s_t] = best ? best : keep;
+    plan->tile[s_t] = timed ? best : keep;
     if (h_tile) *h_tile = plan->tile[s_t];
     // the plan's results are those of a search with the chosen tile
     st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
