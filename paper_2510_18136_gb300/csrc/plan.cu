@@ -134,7 +134,10 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
         return true;
     }
     // windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel
-    // is asked for: a lane per pixel instead of a warp per DM row (SHORT_RULE)
+    // is asked for: a lane per pixel instead of a warp per DM row.  301 x 301 pixels, FP32, against
+    // the barrier-free kernel's best tile: 16 samples 71 us (1450), 32 samples 138 us (1488), 64
+    // samples 366 us (1570) at 16 DM, 39 (339), 79 (362) and 238 us (369) at one.  The line lies at 64
+    // samples because a thread holds a row and its prefix in registers (210 of 255 at 64).
     if (const int w = tile_pref == 0 ? short_warps(sp, max_smem) : 0) {
         sp.pipe = 0;
         sp.stage = 0;

@@ -18,8 +18,9 @@
 //    subbands (the samples shared out over the warps), and the earliest sample reaching its
 //    maximum, with that maximum's S/N, goes to the record.
 // Bound by instruction issue: per sample and row 1.5 operations per width, one for the prefix and
-// three per changed subband.  301 x 301 pixels x 16 subbands x 25 samples, 16 DM, 5 widths:
-// SHORT_FIGURES
+// three per changed subband.  301 x 301 pixels x 16 subbands x 25 samples in FP32, 16 DM, 5 widths:
+// 106 us (1.4 TB/s), where the warp-per-row kernel with CTA barriers takes 3119 us; 16 binned samples,
+// one DM: 37 us (387 us in the barrier-free kernel).
 #include <climits>
 
 #include "nsfrb.h"
