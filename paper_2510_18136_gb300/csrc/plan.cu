@@ -37,6 +37,7 @@ nsfrb_status cuda_check(nsfrb_plan_s *p, cudaError_t e, const char *what) {
 
 cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, cudaStream_t s) {
     if (p.short_w > 0) return launch_search_short(p, smem, s);
+    if (p.mid_w > 0) return launch_search_mid(p, smem, s);
     switch (C) {
         case 1: return launch_search_c1(p, grid, smem, s);
         case 3: return launch_search_c3(p, grid, smem, s);
@@ -145,6 +146,9 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
         smem = short_smem(sp, w);
         return true;
     }
+    // longer ones up to 607 samples: several pixels to a warp (figures and the line between the two
+    // beside the kernel and choose_mid)
+    if (tile_pref == 0 && choose_mid(sp, max_smem, smem)) return true;
     const uintptr_t base = reinterpret_cast<uintptr_t>(sp.cube);
     const int n_t = sp.n_t;
     const int epv = 16 / static_cast<int>(elem_size(sp.dtype));   // samples per 16 bytes
@@ -221,7 +225,7 @@ bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem) {
 void note_tile(nsfrb_plan_s *pl, const SearchParams &sp) {
     pl->last_tile = sp.pipe ? 10 * sp.teams + sp.nb : 0;
     pl->last_tile_st = sp.dtype;
-    pl->last_short = sp.short_w > 0;
+    pl->last_other = sp.short_w > 0 || sp.mid_w > 0;
 }
 
 nsfrb_status ensure_device(nsfrb_plan_s *pl) {
@@ -756,7 +760,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
     if (st == NSFRB_OK) st = nsfrb_last_timing(plan, nullptr, nullptr);
     if (st != NSFRB_OK) return st;
     const int s_t = plan->last_tile_st;
-    if ((plan->last_tile == 0 && !plan->last_short) || s_t < 0) {
+    if ((plan->last_tile == 0 && !plan->last_other) || s_t < 0) {
         if (h_tile) *h_tile = 0;
         return NSFRB_OK;
     }
@@ -765,7 +769,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
     float best_ms = 0.0f;
     bool timed = false;   // best_ms holds a time
     std::vector<float> t(reps);
-    if (plan->last_short) {   // tile 0 is the short-window kernel: a contender of its own
+    if (plan->last_other) {   // tile 0 is the short- or mid-window kernel: a contender of its own
         for (int r = 0; r < reps; ++r) {
             st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
             if (st == NSFRB_OK) st = nsfrb_last_timing(plan, &t[r], nullptr);
