@@ -100,6 +100,8 @@ struct SearchParams {
     int32_t short_w;       // > 0: the short-window kernel with this many warps per CTA
     int32_t mid_w, mid_c, mid_s;   // mid_w > 0: the mid-window kernel, warps per CTA, samples per lane,
                                    // lanes per pixel
+    int32_t wide;          // 1: the wide-window kernel, mid_c samples per lane, mid_s warps per row, nb
+                           // pixel buffers
     // ---- outputs (indexed by absolute pixel)
     PixRec *rec;
     float *full_snr;       // [pix][n_dm][n_w] or nullptr
@@ -176,11 +178,14 @@ cudaError_t prepare_search_long(size_t smem);
 // The short-window kernel: warps per CTA where it applies (0: it does not), and its shared memory.
 int short_warps(const SearchParams &p, int max_smem);
 size_t short_smem(const SearchParams &p, int n_warps);
-cudaError_t launch_search_short(const SearchParams &p, size_t smem, cudaStream_t s);
+cudaError_t launch_search_short(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t prepare_search_short(size_t smem);
 // The mid-window kernel: sets its tile, widths and shared memory in p where it applies.
 bool choose_mid(SearchParams &p, int max_smem, size_t &smem);
-cudaError_t launch_search_mid(const SearchParams &p, size_t smem, cudaStream_t s);
+cudaError_t launch_search_mid(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
+// The wide-window kernel, likewise.
+bool choose_wide(SearchParams &p, int max_smem, size_t &smem);
+cudaError_t launch_search_wide(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 
 // Compaction of per-pixel records into the candidate list ordered by pixel.
 cudaError_t launch_compact(const PixRec *rec, int64_t n_pix, int32_t nx, float thr,

@@ -36,8 +36,9 @@ nsfrb_status cuda_check(nsfrb_plan_s *p, cudaError_t e, const char *what) {
 }
 
 cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, cudaStream_t s) {
-    if (p.short_w > 0) return launch_search_short(p, smem, s);
-    if (p.mid_w > 0) return launch_search_mid(p, smem, s);
+    if (p.short_w > 0) return launch_search_short(p, grid, smem, s);
+    if (p.mid_w > 0) return launch_search_mid(p, grid, smem, s);
+    if (p.wide) return launch_search_wide(p, grid, smem, s);
     switch (C) {
         case 1: return launch_search_c1(p, grid, smem, s);
         case 3: return launch_search_c3(p, grid, smem, s);
@@ -123,8 +124,10 @@ bool tile_is_known(int t) {
 }
 
 bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int tile_pref) {
+    // long windows whose pixels fit in shared memory: several warps to a DM row (figures beside the kernel)
+    if (C == kLongC && choose_wide(sp, max_smem, smem)) return true;
     if (C == kLongC) {
-        // windows beyond the register path: the long-window kernel reads the cube in place; its
+        // other windows beyond the register path: the long-window kernel reads the cube in place; its
         // CTA takes as many warps as their prefix rows fit (the warp count travels in sp.teams)
         sp.pipe = 0;
         sp.stage = 0;

@@ -26,6 +26,7 @@
 // 2940 us (4409); BF16 240 1079 us (4887), 300 1494 us (9300), 600 2515 us (7077).
 #pragma once
 
+#include <algorithm>
 #include <climits>
 
 #include "nsfrb.h"
@@ -105,252 +106,272 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane / S, j = lane % S;   // pixel of the warp's set, chunk of the pixel
     const int n_sub = p.n_sub, n_t = p.n_t, ne = n_sub * n_t;
-    const int64_t it0 = static_cast<int64_t>(blockIdx.x) * PW;
-    const int n_here = static_cast<int>(min(static_cast<int64_t>(PW), p.n_items - it0));
-    const int64_t pix0 = p.pix0 + it0;
-    const unsigned char *src = static_cast<const unsigned char *>(p.cube) + (pix0 - p.cube_pix0) * ne * kEs;
-
-    // ---- samples as stored, tables, 1 / (sigma sqrt(w))
-    if (p.stage == 1) {
-        if (tid == 0) {
-            mbar_init(s_bar, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            fence_proxy_async();
-            const uint32_t bytes = static_cast<uint32_t>(ne * kEs);
-            mbar_expect_tx(s_bar, bytes * static_cast<uint32_t>(n_here));
-            for (int i = 0; i < n_here; ++i)
-                bulk_g2s(s_xs + (size_t)i * lay.pitch * kEs, src + (size_t)i * bytes, bytes, s_bar);
-        }
-    } else {
-        for (int i = 0; i < n_here; ++i)
-            for (int e = tid; e < ne; e += blockDim.x) {
-                const size_t at = (size_t)i * lay.pitch + e, from = (size_t)i * ne + e;
-                if constexpr (ST == 0)
-                    reinterpret_cast<float *>(s_xs)[at] = reinterpret_cast<const float *>(src)[from];
-                else
-                    reinterpret_cast<uint16_t *>(s_xs)[at] = reinterpret_cast<const uint16_t *>(src)[from];
-            }
-    }
+    int64_t n_items = p.n_items;
+    if (p.n_items_dev) n_items = *p.n_items_dev;
+    auto item_pixel = [&](int64_t it) -> int64_t {
+        return p.pix_list ? static_cast<int64_t>(p.pix_list[it]) : p.pix0 + it;
+    };
     const int table_words = p.n_u * kInfo + p.n_deltas + p.n_u * n_sub;
     for (int i = tid; i < table_words; i += blockDim.x) s_table[i] = p.table[i];
     const int32_t *s_info = s_table;
     const int32_t *s_delta = s_table + p.n_u * kInfo;
     const int32_t *s_shift = s_delta + p.n_deltas;
-    for (int i = tid; i < p.n_w * PW; i += blockDim.x) {
-        const float sg = (p.sigma && i % PW < n_here) ? p.sigma[pix0 + i % PW] : p.sigma_default;
-        s_inv[i] = 1.0f / (sg * sqrtf(static_cast<float>(p.widths[i / PW])));
+    if (p.stage == 1 && tid == 0) {
+        mbar_init(s_bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async();
     }
-    __syncthreads();
-    if (p.stage == 1 && !mbar_wait(s_bar, 0)) {
-        if (lane == 0) atomicOr(p.err, ERR_WAIT_TIMEOUT);
-        return;
-    }
+    uint32_t phase = 0;
+    // one set of pixels per CTA, or, where a device count says how many there are (re-scoring), several
+    for (int64_t it0 = static_cast<int64_t>(blockIdx.x) * PW; it0 < n_items;
+         it0 += static_cast<int64_t>(gridDim.x) * PW) {
+        const int n_here = static_cast<int>(min(static_cast<int64_t>(PW), n_items - it0));
+        const unsigned char *cube = static_cast<const unsigned char *>(p.cube);
 
-    // ---- the warp's rows
-    const int n_ua = p.n_u_active;
-    float *Pw = reinterpret_cast<float *>(smem + lay.pbuf) + (size_t)warp * 32 * C;
-    const void *xp = s_xs + (size_t)(q < n_here ? q : 0) * lay.pitch * kEs;
-    const int t0 = j * C;
-    const int u_lo = (warp * n_ua) / n_warps, u_hi = ((warp + 1) * n_ua) / n_warps;
-    float bs = neg_inf();
-    int buw = -1;
-    float2 D[C / 2];
-    int L_prev = -1;
-#pragma unroll 1
-    for (int u = u_lo; u < u_hi; ++u) {
-        const int32_t *info = s_info + u * kInfo;
-        if (u == u_lo) {
-#pragma unroll
-            for (int m = 0; m < C / 2; ++m) D[m] = make_float2(0.0f, 0.0f);
-            const int32_t *sh = s_shift + u * n_sub;
-#pragma unroll 1
-            for (int k = 0; k < n_sub; ++k) mid_acc<C, false, ST>(D, xp, k * n_t + t0 + sh[k]);
+        // ---- samples as stored, 1 / (sigma sqrt(w))
+        if (p.stage == 1) {
+            if (tid == 0) {
+                const uint32_t bytes = static_cast<uint32_t>(ne * kEs);
+                mbar_expect_tx(s_bar, bytes * static_cast<uint32_t>(n_here));
+                for (int i = 0; i < n_here; ++i)
+                    bulk_g2s(s_xs + (size_t)i * lay.pitch * kEs,
+                             cube + (item_pixel(it0 + i) - p.cube_pix0) * static_cast<int64_t>(bytes), bytes, s_bar);
+            }
         } else {
-            const int d0 = info[UI_DOFF], nd = info[UI_ND];
-#pragma unroll 1
-            for (int e = d0; e < d0 + nd; ++e) {
-                const uint32_t pk = static_cast<uint32_t>(s_delta[e]);
-                const int k = pk & 63u, so = (pk >> 6) & 0x1fffu, sn = pk >> 19;
-                const int at = k * n_t + t0;
-                if (sn == so + 1) {
-                    mid_step1<C, ST>(D, xp, at + so);
-                } else {
-                    mid_acc<C, false, ST>(D, xp, at + sn);
-                    mid_acc<C, true, ST>(D, xp, at + so);
+            for (int i = 0; i < n_here; ++i) {
+                const int64_t from = (item_pixel(it0 + i) - p.cube_pix0) * ne;
+                for (int e = tid; e < ne; e += blockDim.x) {
+                    const size_t at = (size_t)i * lay.pitch + e;
+                    if constexpr (ST == 0)
+                        reinterpret_cast<float *>(s_xs)[at] = reinterpret_cast<const float *>(cube)[from + e];
+                    else
+                        reinterpret_cast<uint16_t *>(s_xs)[at] = reinterpret_cast<const uint16_t *>(cube)[from + e];
                 }
             }
         }
-        const int L = n_t - info[UI_SMAX];
-        if (L != L_prev) {
-#pragma unroll
-            for (int m = 0; m < C / 2; ++m) {
-                if (t0 + 2 * m >= L) D[m].x = neg_inf();
-                if (t0 + 2 * m + 1 >= L) D[m].y = neg_inf();
-            }
-            L_prev = L;
+        for (int i = tid; i < p.n_w * PW; i += blockDim.x) {
+            const float sg = (p.sigma && i % PW < n_here) ? p.sigma[item_pixel(it0 + i % PW)] : p.sigma_default;
+            s_inv[i] = 1.0f / (sg * sqrtf(static_cast<float>(p.widths[i / PW])));
         }
-        // ascending widths with a strict '>' keep the smallest index on ties
-        const int uw = u * kMaxW;
-        auto consider = [&](int wi, float m) {
-            const float s = m * s_inv[wi * PW + q];
-            if (s > bs) {
-                bs = s;
-                buw = uw + wi;
-            }
-        };
-        {
-            float2 Lp[C / 2], Hh[SH / 2];
-            const float tot = prefix_pairs<C>(D, Lp);
-            // the last chunk of a pixel ends past its window: its total is -inf or NaN, and with it
-            // the halo that its last lane takes from the next pixel's first
-            halo_pairs<C, SH>(Lp, tot, Hh);
-            float inc = tot;
+        __syncthreads();
+        const int landed = p.stage == 1 ? mbar_wait(s_bar, phase) : 1;
+        phase ^= 1u;
+        if (!__syncthreads_and(landed)) {
+            if (tid == 0) atomicOr(p.err, ERR_WAIT_TIMEOUT);
+            return;
+        }
+
+        // ---- the warp's rows
+        const int n_ua = p.n_u_active;
+        float *Pw = reinterpret_cast<float *>(smem + lay.pbuf) + (size_t)warp * 32 * C;
+        const void *xp = s_xs + (size_t)(q < n_here ? q : 0) * lay.pitch * kEs;
+        const int t0 = j * C;
+        const int u_lo = (warp * n_ua) / n_warps, u_hi = ((warp + 1) * n_ua) / n_warps;
+        float bs = neg_inf();
+        int buw = -1;
+        float2 D[C / 2];
+        int L_prev = -1;
+#pragma unroll 1
+        for (int u = u_lo; u < u_hi; ++u) {
+            const int32_t *info = s_info + u * kInfo;
+            if (u == u_lo) {
 #pragma unroll
-            for (int o = 1; o < S; o <<= 1) {
-                const float y = __shfl_up_sync(kFull, inc, o, S);
-                if (j >= o) inc += y;
+                for (int m = 0; m < C / 2; ++m) D[m] = make_float2(0.0f, 0.0f);
+                const int32_t *sh = s_shift + u * n_sub;
+#pragma unroll 1
+                for (int k = 0; k < n_sub; ++k) mid_acc<C, false, ST>(D, xp, k * n_t + t0 + sh[k]);
+            } else {
+                const int d0 = info[UI_DOFF], nd = info[UI_ND];
+#pragma unroll 1
+                for (int e = d0; e < d0 + nd; ++e) {
+                    const uint32_t pk = static_cast<uint32_t>(s_delta[e]);
+                    const int k = pk & 63u, so = (pk >> 6) & 0x1fffu, sn = pk >> 19;
+                    const int at = k * n_t + t0;
+                    if (sn == so + 1) {
+                        mid_step1<C, ST>(D, xp, at + so);
+                    } else {
+                        mid_acc<C, false, ST>(D, xp, at + sn);
+                        mid_acc<C, true, ST>(D, xp, at + so);
+                    }
+                }
             }
-            float carry = __shfl_up_sync(kFull, inc, 1, S);
-            if (j == 0) carry = 0.0f;
+            const int L = n_t - info[UI_SMAX];
+            if (L != L_prev) {
+#pragma unroll
+                for (int m = 0; m < C / 2; ++m) {
+                    if (t0 + 2 * m >= L) D[m].x = neg_inf();
+                    if (t0 + 2 * m + 1 >= L) D[m].y = neg_inf();
+                }
+                L_prev = L;
+            }
+            // ascending widths with a strict '>' keep the smallest index on ties
+            const int uw = u * kMaxW;
+            auto consider = [&](int wi, float m) {
+                const float s = m * s_inv[wi * PW + q];
+                if (s > bs) {
+                    bs = s;
+                    buw = uw + wi;
+                }
+            };
+            {
+                float2 Lp[C / 2], Hh[SH / 2];
+                const float tot = prefix_pairs<C>(D, Lp);
+                // the last chunk of a pixel ends past its window: its total is -inf or NaN, and with it
+                // the halo that its last lane takes from the next pixel's first
+                halo_pairs<C, SH>(Lp, tot, Hh);
+                float inc = tot;
+#pragma unroll
+                for (int o = 1; o < S; o <<= 1) {
+                    const float y = __shfl_up_sync(kFull, inc, o, S);
+                    if (j >= o) inc += y;
+                }
+                float carry = __shfl_up_sync(kFull, inc, 1, S);
+                if (j == 0) carry = 0.0f;
 #define NSFRB_MID_SMALL(J) \
     if (p.pow2_wi[J] >= 0) consider(p.pow2_wi[J], small_max_pk<C, SH, (1 << J)>(D, Lp, Hh));
-            NSFRB_MID_SMALL(0) NSFRB_MID_SMALL(1) NSFRB_MID_SMALL(2) NSFRB_MID_SMALL(3) NSFRB_MID_SMALL(4)
+                NSFRB_MID_SMALL(0) NSFRB_MID_SMALL(1) NSFRB_MID_SMALL(2) NSFRB_MID_SMALL(3) NSFRB_MID_SMALL(4)
 #undef NSFRB_MID_SMALL
-            store_p<C>(Pw, lane * C, carry, Lp);
-        }
-        __syncwarp();
-        if (p.has_large) {
-            float2 Ps[C / 2];
-            const float2 *src2 = reinterpret_cast<const float2 *>(Pw + q * S * C) + j;
+                store_p<C>(Pw, lane * C, carry, Lp);
+            }
+            __syncwarp();
+            if (p.has_large) {
+                float2 Ps[C / 2];
+                const float2 *src2 = reinterpret_cast<const float2 *>(Pw + q * S * C) + j;
 #pragma unroll
-            for (int m = 0; m < C / 2; ++m) Ps[m] = src2[S * m];
+                for (int m = 0; m < C / 2; ++m) Ps[m] = src2[S * m];
 #define NSFRB_MID_LARGE(J)                                                                     \
     if constexpr ((1 << J) > SH && (1 << J) < S * C) {                                         \
         if (p.pow2_wi[J] >= 0) consider(p.pow2_wi[J], mid_large<C, (1 << J) / (2 * S)>(Ps));  \
     }
-            NSFRB_POW2(NSFRB_MID_LARGE)
+                NSFRB_POW2(NSFRB_MID_LARGE)
 #undef NSFRB_MID_LARGE
-        }
+            }
 #pragma unroll 1
-        for (int g = 0; g < p.n_gen; ++g) {
-            const int wi = p.gen_wi[g], w = p.widths[wi];
-            const float *Pq = Pw + q * S * C;
-            float m = neg_inf();
-            for (int t = j; t + w <= L; t += S) m = fmaxf(m, Pq[t + w] - Pq[t]);
-            const float s = m * s_inv[wi * PW + q];
-            if (s > bs || (s == bs && uw + wi < buw)) {
-                bs = s;
-                buw = uw + wi;
+            for (int g = 0; g < p.n_gen; ++g) {
+                const int wi = p.gen_wi[g], w = p.widths[wi];
+                const float *Pq = Pw + q * S * C;
+                float m = neg_inf();
+                for (int t = j; t + w <= L; t += S) m = fmaxf(m, Pq[t + w] - Pq[t]);
+                const float s = m * s_inv[wi * PW + q];
+                if (s > bs || (s == bs && uw + wi < buw)) {
+                    bs = s;
+                    buw = uw + wi;
+                }
+            }
+            __syncwarp();
+        }
+        // the pixel's best over its lanes: ties go to the smallest row, then width
+#pragma unroll
+        for (int o = S / 2; o > 0; o >>= 1) {
+            const float os = __shfl_xor_sync(kFull, bs, o);
+            const int ob = __shfl_xor_sync(kFull, buw, o);
+            if (os > bs || (os == bs && ob >= 0 && ob < buw)) {
+                bs = os;
+                buw = ob;
             }
         }
-        __syncwarp();
-    }
-    // the pixel's best over its lanes: ties go to the smallest row, then width
-#pragma unroll
-    for (int o = S / 2; o > 0; o >>= 1) {
-        const float os = __shfl_xor_sync(kFull, bs, o);
-        const int ob = __shfl_xor_sync(kFull, buw, o);
-        if (os > bs || (os == bs && ob >= 0 && ob < buw)) {
-            bs = os;
-            buw = ob;
+        if (j == 0) {
+            s_bs[warp * PW + q] = bs;
+            s_buw[warp * PW + q] = buw;
         }
-    }
-    if (j == 0) {
-        s_bs[warp * PW + q] = bs;
-        s_buw[warp * PW + q] = buw;
-    }
-    __syncthreads();
+        __syncthreads();
 
-    // ---- records: a warp per pixel rebuilds its best row
-    for (int i = warp; i < n_here; i += n_warps) {
-        float best = neg_inf();
-        int uw = -1;
-        for (int g = 0; g < n_warps; ++g)
-            if (s_bs[g * PW + i] > best) {
-                best = s_bs[g * PW + i];
-                uw = s_buw[g * PW + i];
-            }
-        PixRec r{neg_inf(), -1, -1, -1};
-        if (uw >= 0) {
-            const int u = uw / kMaxW, wi = uw % kMaxW, w = p.widths[wi];
-            const int32_t *sh = s_shift + u * n_sub;
-            const int L = n_t - s_info[u * kInfo + UI_SMAX];
-            const unsigned char *row = s_xs + (size_t)i * lay.pitch * kEs;
-            const float inv = s_inv[wi * PW + i];
-            // lane l takes samples [l CC, l CC + CC), CC odd: no bank conflicts
-            constexpr int CC = ((S * C + 31) / 32) | 1;
-            const int t1 = lane * CC;
-            float d[CC];
+        // ---- records: a warp per pixel rebuilds its best row
+        for (int i = warp; i < n_here; i += n_warps) {
+            float best = neg_inf();
+            int uw = -1;
+            for (int g = 0; g < n_warps; ++g)
+                if (s_bs[g * PW + i] > best) {
+                    best = s_bs[g * PW + i];
+                    uw = s_buw[g * PW + i];
+                }
+            PixRec r{neg_inf(), -1, -1, -1};
+            if (uw >= 0) {
+                const int u = uw / kMaxW, wi = uw % kMaxW, w = p.widths[wi];
+                const int32_t *sh = s_shift + u * n_sub;
+                const int L = n_t - s_info[u * kInfo + UI_SMAX];
+                const unsigned char *row = s_xs + (size_t)i * lay.pitch * kEs;
+                const float inv = s_inv[wi * PW + i];
+                // lane l takes samples [l CC, l CC + CC), CC odd: no bank conflicts
+                constexpr int CC = ((S * C + 31) / 32) | 1;
+                const int t1 = lane * CC;
+                float d[CC];
 #pragma unroll
-            for (int c = 0; c < CC; ++c) d[c] = 0.0f;
-            if (t1 < L) {
+                for (int c = 0; c < CC; ++c) d[c] = 0.0f;
+                if (t1 < L) {
 #pragma unroll 2
-                for (int k = 0; k < n_sub; ++k) {
-                    const int e = k * n_t + t1 + sh[k];
+                    for (int k = 0; k < n_sub; ++k) {
+                        const int e = k * n_t + t1 + sh[k];
 #pragma unroll
-                    for (int c = 0; c < CC; ++c) {
-                        if constexpr (ST == 0)
-                            d[c] += reinterpret_cast<const float *>(row)[e + c];
-                        else
-                            d[c] += widen16(reinterpret_cast<const uint16_t *>(row)[e + c], ST);
+                        for (int c = 0; c < CC; ++c) {
+                            if constexpr (ST == 0)
+                                d[c] += reinterpret_cast<const float *>(row)[e + c];
+                            else
+                                d[c] += widen16(reinterpret_cast<const uint16_t *>(row)[e + c], ST);
+                        }
                     }
                 }
-            }
-            // w = 1: D in the buffer; else P, with P[t1 + c] kept in d[c]
-            __syncwarp();
-            if (w == 1) {
+                // w = 1: D in the buffer; else P, with P[t1 + c] kept in d[c]
+                __syncwarp();
+                if (w == 1) {
 #pragma unroll
-                for (int c = 0; c < CC; ++c)
-                    if (t1 + c < L) Pw[t1 + c] = d[c];
-            } else {
-                float tot = 0.0f;
+                    for (int c = 0; c < CC; ++c)
+                        if (t1 + c < L) Pw[t1 + c] = d[c];
+                } else {
+                    float tot = 0.0f;
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) {
+                        const float v = t1 + c < L ? d[c] : 0.0f;
+                        d[c] = tot;
+                        tot += v;
+                    }
+                    const float carry = lane_carry(tot, lane);
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) {
+                        d[c] += carry;
+                        if (t1 + c <= L) Pw[t1 + c] = d[c];
+                    }
+                }
+                __syncwarp();
+                float m = neg_inf();
 #pragma unroll
                 for (int c = 0; c < CC; ++c) {
-                    const float v = t1 + c < L ? d[c] : 0.0f;
-                    d[c] = tot;
-                    tot += v;
+                    if (t1 + c + w <= L) {
+                        if (w > 1) d[c] = Pw[t1 + c + w] - d[c];
+                        m = fmaxf(m, d[c]);
+                    }
                 }
-                const float carry = lane_carry(tot, lane);
+                m = warp_max(m);
+                r.snr = m * inv;
+                int at = INT_MAX;
 #pragma unroll
-                for (int c = 0; c < CC; ++c) {
-                    d[c] += carry;
-                    if (t1 + c <= L) Pw[t1 + c] = d[c];
-                }
+                for (int c = CC - 1; c >= 0; --c)
+                    if (t1 + c + w <= L && d[c] * inv == r.snr) at = t1 + c;
+                at = warp_min(at);
+                r.t_idx = at == INT_MAX ? -1 : at;
+                r.dm_idx = s_info[u * kInfo + UI_FIRST_D];
+                r.w_idx = wi;
+                __syncwarp();
             }
-            __syncwarp();
-            float m = neg_inf();
-#pragma unroll
-            for (int c = 0; c < CC; ++c) {
-                if (t1 + c + w <= L) {
-                    if (w > 1) d[c] = Pw[t1 + c + w] - d[c];
-                    m = fmaxf(m, d[c]);
+            if (lane == 0) {
+                const int64_t pix = item_pixel(it0 + i);
+                if (p.bad_pix && p.bad_pix[pix]) {
+                    r = PixRec{neg_inf(), -1, -1, -1};
+                    atomicOr(p.err, ERR_ZERO_MAD);
                 }
+                p.rec[pix] = r;
             }
-            m = warp_max(m);
-            r.snr = m * inv;
-            int at = INT_MAX;
-#pragma unroll
-            for (int c = CC - 1; c >= 0; --c)
-                if (t1 + c + w <= L && d[c] * inv == r.snr) at = t1 + c;
-            at = warp_min(at);
-            r.t_idx = at == INT_MAX ? -1 : at;
-            r.dm_idx = s_info[u * kInfo + UI_FIRST_D];
-            r.w_idx = wi;
-            __syncwarp();
         }
-        if (lane == 0) {
-            if (p.bad_pix && p.bad_pix[pix0 + i]) {
-                r = PixRec{neg_inf(), -1, -1, -1};
-                atomicOr(p.err, ERR_ZERO_MAD);
-            }
-            p.rec[pix0 + i] = r;
-        }
+        fence_proxy_async();
+        __syncthreads();   // everything of this set has been read
     }
 }
 
 template <int C, int S, int ST>
-cudaError_t mid_launch(const SearchParams &p, size_t smem, cudaStream_t s) {
-    const unsigned grid = static_cast<unsigned>((p.n_items + 32 / S - 1) / (32 / S));
+cudaError_t mid_launch(const SearchParams &p, int grid_sm, size_t smem, cudaStream_t s) {
+    // where only the device knows the count, as many CTAs as can run at once (at most) loop over it
+    const int64_t sets = (p.n_items + 32 / S - 1) / (32 / S);
+    const unsigned grid = static_cast<unsigned>(p.n_items_dev ? std::min<int64_t>(sets, 2 * grid_sm) : sets);
     const cudaError_t e = cudaFuncSetAttribute(search_kernel_mid<C, S, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                static_cast<int>(smem));
     if (e != cudaSuccess) return e;
@@ -364,15 +385,15 @@ cudaError_t mid_launch(const SearchParams &p, size_t smem, cudaStream_t s) {
 #define NSFRB_MID_TILES(X) X(22, 4) X(26, 4) X(34, 4) X(22, 8) X(26, 8) X(34, 8) X(22, 16) X(26, 16) X(34, 16) X(38, 16)
 
 #define NSFRB_INSTANTIATE_MID(ST)                                                                     \
-    cudaError_t launch_search_mid_s##ST(const SearchParams &p, size_t smem, cudaStream_t s) {         \
+    cudaError_t launch_search_mid_s##ST(const SearchParams &p, int grid_sm, size_t smem, cudaStream_t s) { \
         switch (100 * p.mid_c + p.mid_s) {                                                            \
             NSFRB_MID_TILES(NSFRB_MID_CASE_##ST)                                                      \
             default:                                                                                  \
                 return cudaErrorInvalidValue;                                                         \
         }                                                                                             \
     }
-#define NSFRB_MID_CASE_0(C, S) case 100 * C + S: return dev::mid_launch<C, S, 0>(p, smem, s);
-#define NSFRB_MID_CASE_1(C, S) case 100 * C + S: return dev::mid_launch<C, S, 1>(p, smem, s);
-#define NSFRB_MID_CASE_2(C, S) case 100 * C + S: return dev::mid_launch<C, S, 2>(p, smem, s);
+#define NSFRB_MID_CASE_0(C, S) case 100 * C + S: return dev::mid_launch<C, S, 0>(p, grid_sm, smem, s);
+#define NSFRB_MID_CASE_1(C, S) case 100 * C + S: return dev::mid_launch<C, S, 1>(p, grid_sm, smem, s);
+#define NSFRB_MID_CASE_2(C, S) case 100 * C + S: return dev::mid_launch<C, S, 2>(p, grid_sm, smem, s);
 
 }  // namespace nsfrb

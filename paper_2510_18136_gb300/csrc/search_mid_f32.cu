@@ -1,17 +1,15 @@
 // Mid-window search kernels for FP32 rows, and the choice among the mid-window tiles.
-#include <algorithm>
-
 #include "search_mid.cuh"
 
 namespace nsfrb {
 
 NSFRB_INSTANTIATE_MID(0)
-cudaError_t launch_search_mid_s1(const SearchParams &, size_t, cudaStream_t);
-cudaError_t launch_search_mid_s2(const SearchParams &, size_t, cudaStream_t);
+cudaError_t launch_search_mid_s1(const SearchParams &, int, size_t, cudaStream_t);
+cudaError_t launch_search_mid_s2(const SearchParams &, int, size_t, cudaStream_t);
 
 bool choose_mid(SearchParams &p, int max_smem, size_t &smem) {
     if (p.n_t <= kShortT || p.full_snr || p.noise_mode != 0 || p.t_wrap || p.t_stride || p.t_off || p.t_off_dev ||
-        p.new_blk || p.pix_list || p.n_items_dev || p.row_len != p.n_t || p.n_u_active < 1)
+        p.new_blk || p.row_len != p.n_t || p.n_u_active < 1)
         return false;
     // Few rows of long FP32 windows stay with the barrier-free kernel where its copies apply: the work is
     // then the copy, which that kernel overlaps with the search (301 x 301 pixels, one DM: 400
@@ -73,10 +71,10 @@ bool choose_mid(SearchParams &p, int max_smem, size_t &smem) {
     return true;
 }
 
-cudaError_t launch_search_mid(const SearchParams &p, size_t smem, cudaStream_t s) {
+cudaError_t launch_search_mid(const SearchParams &p, int grid, size_t smem, cudaStream_t s) {
     if (p.n_items <= 0) return cudaSuccess;
-    if (p.dtype == NSFRB_F32) return launch_search_mid_s0(p, smem, s);
-    return p.dtype == NSFRB_BF16 ? launch_search_mid_s1(p, smem, s) : launch_search_mid_s2(p, smem, s);
+    if (p.dtype == NSFRB_F32) return launch_search_mid_s0(p, grid, smem, s);
+    return p.dtype == NSFRB_BF16 ? launch_search_mid_s1(p, grid, smem, s) : launch_search_mid_s2(p, grid, smem, s);
 }
 
 }  // namespace nsfrb

@@ -21,6 +21,7 @@
 // three per changed subband.  301 x 301 pixels x 16 subbands x 25 samples in FP32, 16 DM, 5 widths:
 // 106 us (1.4 TB/s), where the warp-per-row kernel with CTA barriers takes 3119 us; 16 binned samples,
 // one DM: 37 us (387 us in the barrier-free kernel).
+#include <algorithm>
 #include <climits>
 
 #include "nsfrb.h"
@@ -109,7 +110,8 @@ __device__ __forceinline__ float short_max_any(int w, const float2 (&D)[NT / 2],
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT > 32 ? 256 : 128, NT > 32 ? 1 : 4) search_kernel_short(const __grid_constant__ SearchParams p) {
+__global__ void __launch_bounds__(NT > 32 ? 256 : 128, NT > 32 ? 1 : 4)
+search_kernel_short(const __grid_constant__ SearchParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int n_warps = blockDim.x >> 5;
     const ShortLayout lay = short_layout(p, n_warps);
@@ -122,180 +124,190 @@ __global__ void __launch_bounds__(NT > 32 ? 256 : 128, NT > 32 ? 1 : 4) search_k
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_sub = p.n_sub, n_t = p.n_t, ne = n_sub * n_t;
     const int pitch = short_pitch(n_sub, n_t);
-    const int64_t it0 = static_cast<int64_t>(blockIdx.x) * kShortPix;
-    const int n_here = static_cast<int>(min(static_cast<int64_t>(kShortPix), p.n_items - it0));
-    const int64_t pix0 = p.pix0 + it0;
-
-    // ---- samples, tables, 1 / (sigma sqrt(w))
-    const int64_t el0 = (pix0 - p.cube_pix0) * ne;
-    for (int q = warp; q < kShortPix; q += n_warps) {
-        float *dst = xs + (size_t)q * pitch;
-        if (q >= n_here) {
-            for (int e = lane; e < ne; e += 32) dst[e] = 0.0f;
-        } else if (p.dtype == 0) {
-            const float *src = static_cast<const float *>(p.cube) + el0 + static_cast<int64_t>(q) * ne;
-            for (int e = lane; e < ne; e += 32)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + e)), "l"(src + e) : "memory");
-        } else {
-            const unsigned short *src = static_cast<const unsigned short *>(p.cube) + el0 + static_cast<int64_t>(q) * ne;
-#pragma unroll 8
-            for (int e = lane; e < ne; e += 32) dst[e] = widen16(src[e], p.dtype);
-        }
-    }
-    for (int i = tid; i < kShortPad; i += blockDim.x) xs[(size_t)kShortPix * pitch + i] = 0.0f;
+    int64_t n_items = p.n_items;
+    if (p.n_items_dev) n_items = *p.n_items_dev;
+    auto item_pixel = [&](int64_t it) -> int64_t {
+        return p.pix_list ? static_cast<int64_t>(p.pix_list[it]) : p.pix0 + it;
+    };
     const int table_words = p.n_u * kInfo + p.n_deltas + p.n_u * n_sub;
     for (int i = tid; i < table_words; i += blockDim.x) s_table[i] = p.table[i];
     const int32_t *s_info = s_table;
     const int32_t *s_delta = s_table + p.n_u * kInfo;
     const int32_t *s_shift = s_delta + p.n_deltas;
-    {
-        const float sg = (p.sigma && lane < n_here) ? p.sigma[pix0 + lane] : p.sigma_default;
-        for (int wi = warp; wi < p.n_w; wi += n_warps)
-            s_inv[wi * kShortPix + lane] = 1.0f / (sg * sqrtf(static_cast<float>(p.widths[wi])));
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
+    // one set of pixels per CTA, or, where a device count says how many there are (re-scoring), several
+    for (int64_t it0 = static_cast<int64_t>(blockIdx.x) * kShortPix; it0 < n_items;
+         it0 += static_cast<int64_t>(gridDim.x) * kShortPix) {
+        const int n_here = static_cast<int>(min(static_cast<int64_t>(kShortPix), n_items - it0));
 
-    // ---- the warp's rows of all 32 pixels
-    const int n_ua = p.n_u_active;
-    const int n_grp = min(n_warps, n_ua);
-    float bs = neg_inf();
-    int buw = -1;
-    if (warp < n_grp) {
-        const int u_lo = (warp * n_ua) / n_grp, u_hi = ((warp + 1) * n_ua) / n_grp;
-        const float *xp = xs + (size_t)lane * pitch;
-        float2 D[NT / 2];
-        int L_prev = NT + 1;
-#pragma unroll 1
-        for (int u = u_lo; u < u_hi; ++u) {
-            const int32_t *info = s_info + u * kInfo;
-            if (u == u_lo) {
-#pragma unroll
-                for (int m = 0; m < NT / 2; ++m) D[m] = make_float2(0.0f, 0.0f);
-                const int32_t *sh = s_shift + u * n_sub;
-#pragma unroll 1
-                for (int k = 0; k < n_sub; ++k) {
-                    const float *x = xp + k * n_t + sh[k];
-#pragma unroll
-                    for (int m = 0; m < NT / 2; ++m) D[m] = add2(D[m], make_float2(x[2 * m], x[2 * m + 1]));
-                }
+        // ---- samples, 1 / (sigma sqrt(w))
+        for (int q = warp; q < kShortPix; q += n_warps) {
+            float *dst = xs + (size_t)q * pitch;
+            const int64_t from = q < n_here ? (item_pixel(it0 + q) - p.cube_pix0) * ne : 0;
+            if (q >= n_here) {
+                for (int e = lane; e < ne; e += 32) dst[e] = 0.0f;
+            } else if (p.dtype == 0) {
+                const float *src = static_cast<const float *>(p.cube) + from;
+                for (int e = lane; e < ne; e += 32)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + e)), "l"(src + e) : "memory");
             } else {
-                const int d0 = info[UI_DOFF], nd = info[UI_ND];
+                const unsigned short *src = static_cast<const unsigned short *>(p.cube) + from;
+#pragma unroll 8
+                for (int e = lane; e < ne; e += 32) dst[e] = widen16(src[e], p.dtype);
+            }
+        }
+        for (int i = tid; i < kShortPad; i += blockDim.x) xs[(size_t)kShortPix * pitch + i] = 0.0f;
+        {
+            const float sg = (p.sigma && lane < n_here) ? p.sigma[item_pixel(it0 + lane)] : p.sigma_default;
+            for (int wi = warp; wi < p.n_w; wi += n_warps)
+                s_inv[wi * kShortPix + lane] = 1.0f / (sg * sqrtf(static_cast<float>(p.widths[wi])));
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+
+        // ---- the warp's rows of all 32 pixels
+        const int n_ua = p.n_u_active;
+        const int n_grp = min(n_warps, n_ua);
+        float bs = neg_inf();
+        int buw = -1;
+        if (warp < n_grp) {
+            const int u_lo = (warp * n_ua) / n_grp, u_hi = ((warp + 1) * n_ua) / n_grp;
+            const float *xp = xs + (size_t)lane * pitch;
+            float2 D[NT / 2];
+            int L_prev = NT + 1;
 #pragma unroll 1
-                for (int e = d0; e < d0 + nd; ++e) {
-                    const uint32_t pk = static_cast<uint32_t>(s_delta[e]);
-                    const int k = pk & 63u, so = (pk >> 6) & 0x1fffu, sn = pk >> 19;
-                    const float *xo = xp + k * n_t + so;
-                    if (sn == so + 1) {   // both values from one read of the row
-                        float a = xo[0];
+            for (int u = u_lo; u < u_hi; ++u) {
+                const int32_t *info = s_info + u * kInfo;
+                if (u == u_lo) {
 #pragma unroll
-                        for (int m = 0; m < NT / 2; ++m) {
-                            const float b = xo[2 * m + 1], c = xo[2 * m + 2];
-                            D[m] = add2(D[m], make_float2(b - a, c - b));
-                            a = c;
+                    for (int m = 0; m < NT / 2; ++m) D[m] = make_float2(0.0f, 0.0f);
+                    const int32_t *sh = s_shift + u * n_sub;
+#pragma unroll 1
+                    for (int k = 0; k < n_sub; ++k) {
+                        const float *x = xp + k * n_t + sh[k];
+#pragma unroll
+                        for (int m = 0; m < NT / 2; ++m) D[m] = add2(D[m], make_float2(x[2 * m], x[2 * m + 1]));
+                    }
+                } else {
+                    const int d0 = info[UI_DOFF], nd = info[UI_ND];
+#pragma unroll 1
+                    for (int e = d0; e < d0 + nd; ++e) {
+                        const uint32_t pk = static_cast<uint32_t>(s_delta[e]);
+                        const int k = pk & 63u, so = (pk >> 6) & 0x1fffu, sn = pk >> 19;
+                        const float *xo = xp + k * n_t + so;
+                        if (sn == so + 1) {   // both values from one read of the row
+                            float a = xo[0];
+#pragma unroll
+                            for (int m = 0; m < NT / 2; ++m) {
+                                const float b = xo[2 * m + 1], c = xo[2 * m + 2];
+                                D[m] = add2(D[m], make_float2(b - a, c - b));
+                                a = c;
+                            }
+                        } else {
+                            const float *xn = xp + k * n_t + sn;
+#pragma unroll
+                            for (int m = 0; m < NT / 2; ++m)
+                                D[m] = sub2(add2(D[m], make_float2(xn[2 * m], xn[2 * m + 1])),
+                                            make_float2(xo[2 * m], xo[2 * m + 1]));
                         }
-                    } else {
-                        const float *xn = xp + k * n_t + sn;
+                    }
+                }
+                const int L = n_t - info[UI_SMAX];
+                if (L != L_prev) {
 #pragma unroll
-                        for (int m = 0; m < NT / 2; ++m)
-                            D[m] = sub2(add2(D[m], make_float2(xn[2 * m], xn[2 * m + 1])),
-                                        make_float2(xo[2 * m], xo[2 * m + 1]));
+                    for (int m = 0; m < NT / 2; ++m) {
+                        if (2 * m >= L) D[m].x = neg_inf();
+                        if (2 * m + 1 >= L) D[m].y = neg_inf();
+                    }
+                    L_prev = L;
+                }
+                float2 P[NT / 2 + 1];
+                float run = 0.0f;
+                P[0].x = 0.0f;
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    run += pget(D, t);
+                    pset(P, t + 1, run);
+                }
+#pragma unroll 1
+                for (int wi = 0; wi < p.n_w; ++wi) {
+                    const int w = p.widths[wi];
+                    if (w > L) break;
+                    const float s = short_max_any<NT>(w, D, P) * s_inv[wi * kShortPix + lane];
+                    if (s > bs) {   // ascending rows and widths: ties keep the smallest
+                        bs = s;
+                        buw = u * kMaxW + wi;
                     }
                 }
             }
-            const int L = n_t - info[UI_SMAX];
-            if (L != L_prev) {
-#pragma unroll
-                for (int m = 0; m < NT / 2; ++m) {
-                    if (2 * m >= L) D[m].x = neg_inf();
-                    if (2 * m + 1 >= L) D[m].y = neg_inf();
-                }
-                L_prev = L;
-            }
-            float2 P[NT / 2 + 1];
-            float run = 0.0f;
-            P[0].x = 0.0f;
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                run += pget(D, t);
-                pset(P, t + 1, run);
-            }
-#pragma unroll 1
-            for (int wi = 0; wi < p.n_w; ++wi) {
-                const int w = p.widths[wi];
-                if (w > L) break;
-                const float s = short_max_any<NT>(w, D, P) * s_inv[wi * kShortPix + lane];
-                if (s > bs) {   // ascending rows and widths: ties keep the smallest
-                    bs = s;
-                    buw = u * kMaxW + wi;
-                }
-            }
+            s_bs[warp * kShortPix + lane] = bs;
+            s_buw[warp * kShortPix + lane] = buw;
         }
-        s_bs[warp * kShortPix + lane] = bs;
-        s_buw[warp * kShortPix + lane] = buw;
-    }
-    __syncthreads();
+        __syncthreads();
 
-    // ---- the pixel's best row, rebuilt from all subbands: warp q takes samples q, q + n_warps, ...
-    for (int g = 0; g < n_grp; ++g) {
-        const float s = s_bs[g * kShortPix + lane];
-        if (g == 0 || s > bs) {
-            bs = s;
-            buw = s_buw[g * kShortPix + lane];
-        }
-    }
-    if (n_grp == 0) buw = -1;
-    const bool any = buw >= 0;
-    const int bu = any ? buw / kMaxW : 0, bwi = any ? buw % kMaxW : 0;
-    const int L = n_t - s_info[bu * kInfo + UI_SMAX];
-    constexpr int kW = NT > 32 ? 8 : 4;          // = n_warps
-    constexpr int kMine = (NT + kW - 1) / kW;   // samples per thread
-    float d[kMine];
-#pragma unroll
-    for (int j = 0; j < kMine; ++j) d[j] = 0.0f;
-    if (any) {
-        const float *xp = xs + (size_t)lane * pitch + warp;
-        const int32_t *sh = s_shift + bu * n_sub;
-#pragma unroll 2
-        for (int k = 0; k < n_sub; ++k) {
-            const float *x = xp + k * n_t + sh[k];
-#pragma unroll
-            for (int j = 0; j < kMine; ++j) d[j] += x[j * kW];
-        }
-    }
-    __syncthreads();   // the last reads of the samples: their words take the rows now
-#pragma unroll
-    for (int j = 0; j < kMine; ++j)
-        if (warp + j * kW < n_t) xs[(warp + j * kW) * kShortPix + lane] = d[j];
-    __syncthreads();
-    if (warp != 0 || lane >= n_here) return;
-    PixRec r{neg_inf(), -1, -1, -1};
-    if (any) {
-        const int w = p.widths[bwi];
-        const float inv = s_inv[bwi * kShortPix + lane];
-        float *col = xs + lane;   // D[t] at col[t * 32]; P[t] in its place for w > 1
-        if (w > 1) {
-            float run = 0.0f;
-            for (int t = 0; t <= L; ++t) {
-                const float v = t < L ? col[t * kShortPix] : 0.0f;
-                col[t * kShortPix] = run;
-                run += v;
+        // ---- the pixel's best row, rebuilt from all subbands: warp q takes samples q, q + n_warps, ...
+        for (int g = 0; g < n_grp; ++g) {
+            const float s = s_bs[g * kShortPix + lane];
+            if (g == 0 || s > bs) {
+                bs = s;
+                buw = s_buw[g * kShortPix + lane];
             }
         }
-        auto box = [&](int t) { return w == 1 ? col[t * kShortPix] : col[(t + w) * kShortPix] - col[t * kShortPix]; };
-        float m = neg_inf();
-        for (int t = 0; t + w <= L; ++t) m = fmaxf(m, box(t));
-        r.snr = m * inv;
-        for (int t = L - w; t >= 0; --t)
-            if (box(t) * inv == r.snr) r.t_idx = t;
-        r.dm_idx = s_info[bu * kInfo + UI_FIRST_D];
-        r.w_idx = bwi;
+        if (n_grp == 0) buw = -1;
+        const bool any = buw >= 0;
+        const int bu = any ? buw / kMaxW : 0, bwi = any ? buw % kMaxW : 0;
+        const int L = n_t - s_info[bu * kInfo + UI_SMAX];
+        constexpr int kW = NT > 32 ? 8 : 4;          // = n_warps
+        constexpr int kMine = (NT + kW - 1) / kW;   // samples per thread
+        float d[kMine];
+#pragma unroll
+        for (int j = 0; j < kMine; ++j) d[j] = 0.0f;
+        if (any) {
+            const float *xp = xs + (size_t)lane * pitch + warp;
+            const int32_t *sh = s_shift + bu * n_sub;
+#pragma unroll 2
+            for (int k = 0; k < n_sub; ++k) {
+                const float *x = xp + k * n_t + sh[k];
+#pragma unroll
+                for (int j = 0; j < kMine; ++j) d[j] += x[j * kW];
+            }
+        }
+        __syncthreads();   // the last reads of the samples: their words take the rows now
+#pragma unroll
+        for (int j = 0; j < kMine; ++j)
+            if (warp + j * kW < n_t) xs[(warp + j * kW) * kShortPix + lane] = d[j];
+        __syncthreads();
+        if (warp == 0 && lane < n_here) {
+            PixRec r{neg_inf(), -1, -1, -1};
+            if (any) {
+                const int w = p.widths[bwi];
+                const float inv = s_inv[bwi * kShortPix + lane];
+                float *col = xs + lane;   // D[t] at col[t * 32]; P[t] in its place for w > 1
+                if (w > 1) {
+                    float run = 0.0f;
+                    for (int t = 0; t <= L; ++t) {
+                        const float v = t < L ? col[t * kShortPix] : 0.0f;
+                        col[t * kShortPix] = run;
+                        run += v;
+                    }
+                }
+                auto box = [&](int t) { return w == 1 ? col[t * kShortPix] : col[(t + w) * kShortPix] - col[t * kShortPix]; };
+                float m = neg_inf();
+                for (int t = 0; t + w <= L; ++t) m = fmaxf(m, box(t));
+                r.snr = m * inv;
+                for (int t = L - w; t >= 0; --t)
+                    if (box(t) * inv == r.snr) r.t_idx = t;
+                r.dm_idx = s_info[bu * kInfo + UI_FIRST_D];
+                r.w_idx = bwi;
+            }
+            const int64_t pix = item_pixel(it0 + lane);
+            if (p.bad_pix && p.bad_pix[pix]) {
+                r = PixRec{neg_inf(), -1, -1, -1};
+                atomicOr(p.err, ERR_ZERO_MAD);
+            }
+            p.rec[pix] = r;
+        }
+        __syncthreads();   // everything of this set has been read
     }
-    if (p.bad_pix && p.bad_pix[pix0 + lane]) {
-        r = PixRec{neg_inf(), -1, -1, -1};
-        atomicOr(p.err, ERR_ZERO_MAD);
-    }
-    p.rec[pix0 + lane] = r;
 }
 
 }  // namespace dev
@@ -304,7 +316,7 @@ __global__ void __launch_bounds__(NT > 32 ? 256 : 128, NT > 32 ? 1 : 4) search_k
 // pixel-major cube with a known noise, up to 64 samples, whose tile fits in shared memory.
 int short_warps(const SearchParams &p, int max_smem) {
     if (p.n_t > kShortT || p.full_snr || p.noise_mode != 0 || p.t_wrap || p.t_stride || p.t_off || p.t_off_dev ||
-        p.new_blk || p.pix_list || p.n_items_dev || p.row_len != p.n_t)
+        p.new_blk || p.row_len != p.n_t)
         return 0;
     const int w = p.n_t > 32 ? 8 : 4;
     return dev::short_layout(p, w).total <= static_cast<size_t>(max_smem) ? w : 0;
@@ -312,8 +324,10 @@ int short_warps(const SearchParams &p, int max_smem) {
 
 size_t short_smem(const SearchParams &p, int n_warps) { return dev::short_layout(p, n_warps).total; }
 
-cudaError_t launch_search_short(const SearchParams &p, size_t smem, cudaStream_t s) {
-    const unsigned grid = static_cast<unsigned>((p.n_items + dev::kShortPix - 1) / dev::kShortPix);
+cudaError_t launch_search_short(const SearchParams &p, int grid_sm, size_t smem, cudaStream_t s) {
+    // where only the device knows the count, as many CTAs as can run at once (at most) loop over it
+    const int64_t sets = (p.n_items + dev::kShortPix - 1) / dev::kShortPix;
+    const unsigned grid = static_cast<unsigned>(p.n_items_dev ? std::min<int64_t>(sets, 4 * grid_sm) : sets);
     const unsigned threads = 32u * static_cast<unsigned>(p.short_w);
     if (p.n_items <= 0) return cudaSuccess;
     if (p.n_t <= 16)
