@@ -306,16 +306,21 @@ __device__ __forceinline__ void lane_halo(const float (&Lp)[C + 1], float tot, i
     }
 }
 
+// Warp reductions in one instruction (redux; the FP32 maximum is sm_100+ and ignores NaN like max.f32).
 __device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFull, v, o));
-    return v;
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
 }
 
-__device__ __forceinline__ int warp_min(int v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(kFull, v, o));
-    return v;
+__device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(kFull, v); }
+
+// The warp's largest S/N and the smallest width index that has it (-1 where no lane has one), on
+// every lane.  An S/N is -inf (width -1) or a number, never NaN.
+__device__ __forceinline__ void warp_argmax(float &s, int &w) {
+    const float m = warp_max(s);
+    w = static_cast<int>(__reduce_min_sync(kFull, s == m ? static_cast<unsigned>(w) : 0xffffffffu));
+    s = m;
 }
 
 // ------------------------------------------------------------------ even chunks: sample pairs
@@ -827,15 +832,7 @@ if constexpr (FULL) {                                                           
         if constexpr (FULL) full_store_row(p, info, pix, lane, fs, ft);
 
         // warp arg-max over (S/N, width index)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float os = __shfl_xor_sync(kFull, ls, o);
-            const int ow = __shfl_xor_sync(kFull, lw, o);
-            if (os > ls || (os == ls && ow < lw && ow >= 0)) {
-                ls = os;
-                lw = ow;
-            }
-        }
+        warp_argmax(ls, lw);
         if (ls > bsnr) {
             // earliest sample reaching this S/N, re-evaluated exactly as above
             // (the prefix and halo are rebuilt from D: same operations, same values)
@@ -1142,15 +1139,7 @@ __device__ __forceinline__ PixRec search_rows_even(const SearchParams &p, const 
         if (__any_sync(kFull, ls > bsnr)) {
             const float ls_own = ls;
             const int lw_own = lw;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float os = __shfl_xor_sync(kFull, ls, o);
-                const int ow = __shfl_xor_sync(kFull, lw, o);
-                if (os > ls || (os == ls && ow < lw && ow >= 0)) {
-                    ls = os;
-                    lw = ow;
-                }
-            }
+            warp_argmax(ls, lw);
             if (ls > bsnr) {
                 // earliest sample reaching this S/N, re-evaluated with the same operations on the
                 // lanes whose own best it is

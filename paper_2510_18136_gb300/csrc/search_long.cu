@@ -303,15 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_long(const __grid_c
             }
             // warp arg-max over (S/N, width index), only when some lane beats the warp's best
             if (__any_sync(kFull, ls > bsnr)) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float os = __shfl_xor_sync(kFull, ls, o);
-                    const int ow = __shfl_xor_sync(kFull, lw, o);
-                    if (os > ls || (os == ls && ow < lw && ow >= 0)) {
-                        ls = os;
-                        lw = ow;
-                    }
-                }
+                warp_argmax(ls, lw);
                 if (ls > bsnr) {
                     const int w = p.widths[lw];
                     const int tl = masked ? max(0, L - w - p.new_blk + 1) : 0;
