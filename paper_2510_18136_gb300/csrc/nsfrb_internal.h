@@ -102,6 +102,7 @@ struct SearchParams {
                                    // lanes per pixel
     int32_t wide;          // 1: the wide-window kernel, mid_c samples per lane, mid_s warps per row, nb
                            // pixel buffers
+    int32_t team;          // 1: the team kernel, mid_c samples per lane, teams of mid_s warps
     // ---- outputs (indexed by absolute pixel)
     PixRec *rec;
     float *full_snr;       // [pix][n_dm][n_w] or nullptr
@@ -183,9 +184,11 @@ cudaError_t prepare_search_short(size_t smem);
 // The mid-window kernel: sets its tile, widths and shared memory in p where it applies.
 bool choose_mid(SearchParams &p, int max_smem, size_t &smem);
 cudaError_t launch_search_mid(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
-// The wide-window kernel, likewise.
+// The wide-window and team kernels, likewise.
 bool choose_wide(SearchParams &p, int max_smem, size_t &smem);
 cudaError_t launch_search_wide(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
+bool choose_team(SearchParams &p, int max_smem, size_t &smem);
+cudaError_t launch_search_team(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 
 // Compaction of per-pixel records into the candidate list ordered by pixel.
 cudaError_t launch_compact(const PixRec *rec, int64_t n_pix, int32_t nx, float thr,

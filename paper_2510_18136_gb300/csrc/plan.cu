@@ -39,6 +39,7 @@ cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, c
     if (p.short_w > 0) return launch_search_short(p, grid, smem, s);
     if (p.mid_w > 0) return launch_search_mid(p, grid, smem, s);
     if (p.wide) return launch_search_wide(p, grid, smem, s);
+    if (p.team) return launch_search_team(p, grid, smem, s);
     switch (C) {
         case 1: return launch_search_c1(p, grid, smem, s);
         case 3: return launch_search_c3(p, grid, smem, s);
@@ -152,6 +153,8 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
     // longer ones up to 607 samples: several pixels to a warp (figures and the line between the two
     // beside the kernel and choose_mid)
     if (tile_pref == 0 && choose_mid(sp, max_smem, smem)) return true;
+    // and up to 1215 samples: the barrier-free search with more warps (figures beside the kernel)
+    if (tile_pref == 0 && choose_team(sp, max_smem, smem)) return true;
     const uintptr_t base = reinterpret_cast<uintptr_t>(sp.cube);
     const int n_t = sp.n_t;
     const int epv = 16 / static_cast<int>(elem_size(sp.dtype));   // samples per 16 bytes
@@ -228,7 +231,7 @@ bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem) {
 void note_tile(nsfrb_plan_s *pl, const SearchParams &sp) {
     pl->last_tile = sp.pipe ? 10 * sp.teams + sp.nb : 0;
     pl->last_tile_st = sp.dtype;
-    pl->last_other = sp.short_w > 0 || sp.mid_w > 0;
+    pl->last_other = sp.short_w > 0 || sp.mid_w > 0 || sp.team;
 }
 
 nsfrb_status ensure_device(nsfrb_plan_s *pl) {
@@ -772,7 +775,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
     float best_ms = 0.0f;
     bool timed = false;   // best_ms holds a time
     std::vector<float> t(reps);
-    if (plan->last_other) {   // tile 0 is the short- or mid-window kernel: a contender of its own
+    if (plan->last_other) {   // tile 0 is another kernel: a contender of its own
         for (int r = 0; r < reps; ++r) {
             st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
             if (st == NSFRB_OK) st = nsfrb_last_timing(plan, &t[r], nullptr);

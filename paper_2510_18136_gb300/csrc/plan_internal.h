@@ -27,7 +27,7 @@ struct nsfrb_plan_s {
     // searched rows (FP32, BF16, FP16); 0 = the first of the default order that fits
     int32_t tile[3] = {0, 0, 0};
     int32_t last_tile = 0, last_tile_st = -1;   // tile and storage type of the last search launch
-    bool last_other = false;                    // it ran the short- or mid-window kernel
+    bool last_other = false;                    // it ran another kernel than the barrier-free or barrier one
 
     // device state (allocated on first use)
     bool dev_ready = false;
