@@ -20,7 +20,8 @@ __global__ void __launch_bounds__(kCompactBlock) count_kernel(const PixRec *rec,
 __global__ void __launch_bounds__(kCompactBlock) scatter_kernel(const PixRec *rec, int64_t n, int32_t nx,
                                                                float thr, const int32_t *counts,
                                                                int32_t n_blocks, CandRec *out,
-                                                               int32_t *n_out) {
+                                                               int32_t *n_out, const int32_t *err,
+                                                               HostResult *host) {
     __shared__ int32_t s_warp[kCompactBlock / 32];
     __shared__ int32_t s_off;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -41,13 +42,18 @@ __global__ void __launch_bounds__(kCompactBlock) scatter_kernel(const PixRec *re
     const int32_t pos = s_off + before + __popc(bal & ((1u << lane) - 1u));
     if (flag) {
         const PixRec r = rec[i];
-        out[pos] = CandRec{static_cast<int32_t>(i / nx), static_cast<int32_t>(i % nx), r.dm_idx, r.w_idx,
-                           r.t_idx, r.snr};
+        const CandRec c{static_cast<int32_t>(i / nx), static_cast<int32_t>(i % nx), r.dm_idx, r.w_idx, r.t_idx, r.snr};
+        out[pos] = c;
+        if (host && pos < kHostCands) host->cand[pos] = c;
     }
     if (blockIdx.x == n_blocks - 1 && threadIdx.x == 0) {
         int32_t tot = 0;
         for (int w = 0; w < kCompactBlock / 32; ++w) tot += s_warp[w];
         *n_out = s_off + tot;
+        if (host) {
+            host->err = *err;
+            host->n = s_off + tot;
+        }
     }
 }
 
@@ -65,11 +71,13 @@ __global__ void rescore_select_kernel(const PixRec *rec, int64_t n, float thr, f
 }  // namespace
 
 cudaError_t launch_compact(const PixRec *rec, int64_t n_pix, int32_t nx, float thr, int32_t *block_counts,
-                           int32_t n_blocks, CandRec *out, int32_t *n_out, cudaStream_t s) {
+                           int32_t n_blocks, CandRec *out, int32_t *n_out, const int32_t *err, HostResult *host,
+                           cudaStream_t s) {
     count_kernel<<<n_blocks, kCompactBlock, 0, s>>>(rec, n_pix, thr, block_counts);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    scatter_kernel<<<n_blocks, kCompactBlock, 0, s>>>(rec, n_pix, nx, thr, block_counts, n_blocks, out, n_out);
+    scatter_kernel<<<n_blocks, kCompactBlock, 0, s>>>(rec, n_pix, nx, thr, block_counts, n_blocks, out, n_out, err,
+                                                     host);
     return cudaGetLastError();
 }
 

@@ -190,10 +190,19 @@ cudaError_t launch_search_wide(const SearchParams &p, int grid, size_t smem, cud
 bool choose_team(SearchParams &p, int max_smem, size_t &smem);
 cudaError_t launch_search_team(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 
-// Compaction of per-pixel records into the candidate list ordered by pixel.
+// What a search leaves in pinned, mapped host memory: its error word, the number of candidates and the
+// first of them, so that reading a short list after the search is no copy of its own.
+constexpr int kHostCands = 1024;
+struct HostResult {
+    int32_t err, n, pad[2];
+    CandRec cand[kHostCands];
+};
+
+// Compaction of per-pixel records into the candidate list ordered by pixel; host (or null) also gets
+// the error word, the count and the first kHostCands candidates.
 cudaError_t launch_compact(const PixRec *rec, int64_t n_pix, int32_t nx, float thr,
                            int32_t *block_counts, int32_t n_blocks, CandRec *out,
-                           int32_t *n_out, cudaStream_t s);
+                           int32_t *n_out, const int32_t *err, HostResult *host, cudaStream_t s);
 // Pixels whose S/N lies within +-eps of the threshold -> list (unordered).
 cudaError_t launch_rescore_select(const PixRec *rec, int64_t n_pix, float thr, float eps,
                                   int32_t *list, int32_t *n_list, cudaStream_t s);

@@ -281,8 +281,12 @@ nsfrb_status ensure_device(nsfrb_plan_s *pl) {
     if ((st = cuda_check(pl, cudaMemset(pl->d_counts, 0, (pl->n_blocks + 4) * sizeof(int32_t)), "memset")))
         return st;
     if ((st = cuda_check(pl, prepare_search(pl->C, pl->max_smem), "smem attribute")) != NSFRB_OK) return st;
-    if ((st = cuda_check(pl, cudaEventCreateWithFlags(&pl->done, cudaEventDisableTiming), "event")) ||
-        (st = cuda_check(pl, cudaEventCreate(&pl->t_start), "event")) ||
+    if (cudaHostAlloc(reinterpret_cast<void **>(&pl->h_res), sizeof(HostResult), cudaHostAllocMapped | cudaHostAllocPortable) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        pl->h_res = nullptr;
+    }
+    if ((st = cuda_check(pl, cudaEventCreate(&pl->t_start), "event")) ||
         (st = cuda_check(pl, cudaEventCreate(&pl->t_search), "event")) ||
         (st = cuda_check(pl, cudaEventCreate(&pl->t_end), "event")))
         return st;
@@ -381,10 +385,9 @@ nsfrb_status queue_finish(nsfrb_plan_s *pl, cudaStream_t s) {
     if (st != NSFRB_OK) return st;
     st = cuda_check(pl,
                                  launch_compact(pl->d_rec, n_pix, c.nx, c.threshold, pl->d_counts, pl->n_blocks,
-                                                pl->d_cand, pl->d_ncand, s),
+                                                pl->d_cand, pl->d_ncand, pl->d_err, pl->h_res, s),
                                  "compaction");
     if (st != NSFRB_OK) return st;
-    if ((st = cuda_check(pl, cudaEventRecord(pl->done, s), "event record")) != NSFRB_OK) return st;
     if ((st = cuda_check(pl, cudaEventRecord(pl->t_end, s), "event record")) != NSFRB_OK) return st;
     pl->searched = true;
     return NSFRB_OK;
@@ -393,7 +396,30 @@ nsfrb_status queue_finish(nsfrb_plan_s *pl, cudaStream_t s) {
 nsfrb_status wait_done(nsfrb_plan_s *pl) {
     if (pl->latched != NSFRB_OK) return fail(pl, pl->latched, "plan has a latched CUDA error");
     if (!pl->searched) return fail(pl, NSFRB_ENOTREADY, "no search has been run on this plan");
-    return cuda_check(pl, cudaEventSynchronize(pl->done), "wait for search");
+    return cuda_check(pl, cudaEventSynchronize(pl->t_end), "wait for search");
+}
+
+// The finished search's candidates: from the pinned result where they all lie there, else copied.
+nsfrb_status read_candidates(nsfrb_plan_s *pl, nsfrb_candidate *h_out, int32_t cap, int32_t *n_total) {
+    nsfrb_status st;
+    int32_t hdr[2] = {0, 0};   // error word, candidates
+    if (pl->h_res) {
+        hdr[0] = pl->h_res->err;
+        hdr[1] = pl->h_res->n;
+    } else if ((st = cuda_check(pl, cudaMemcpy(hdr, pl->d_err, sizeof(hdr), cudaMemcpyDeviceToHost), "copy")) != NSFRB_OK) {
+        return st;
+    }
+    *n_total = hdr[1];
+    const int32_t n = std::min(hdr[1], cap);
+    if (n > 0 && pl->h_res && n <= kHostCands)
+        std::memcpy(h_out, pl->h_res->cand, sizeof(CandRec) * n);
+    else if (n > 0 && (st = cuda_check(pl, cudaMemcpy(h_out, pl->d_cand, sizeof(CandRec) * n, cudaMemcpyDeviceToHost),
+                                       "copy candidates")) != NSFRB_OK)
+        return st;
+    if (hdr[0] & ERR_WAIT_TIMEOUT) return fail(pl, NSFRB_ETIMEOUT, "a bulk copy into shared memory timed out");
+    if (hdr[0] & ERR_ZERO_MAD) return fail(pl, NSFRB_EINVAL, "zero MAD in at least one (pixel, subband) row");
+    if (hdr[1] > cap) return fail(pl, NSFRB_ETRUNC, "more candidates than capacity");
+    return NSFRB_OK;
 }
 
 }  // namespace nsfrb
@@ -667,19 +693,7 @@ nsfrb_status nsfrb_candidates(nsfrb_plan_t plan, nsfrb_candidate *h_out, int32_t
     if (!plan || !n_total || cap < 0 || (cap > 0 && !h_out)) return fail(plan, NSFRB_EINVAL, "bad argument");
     nsfrb_status st = wait_done(plan);
     if (st != NSFRB_OK) return st;
-    int32_t hdr[2] = {0, 0};   // err, n_cand
-    if ((st = cuda_check(plan, cudaMemcpy(hdr, plan->d_err, sizeof(hdr), cudaMemcpyDeviceToHost), "copy")) != NSFRB_OK)
-        return st;
-    *n_total = hdr[1];
-    const int32_t n = std::min(hdr[1], cap);
-    if (n > 0 &&
-        (st = cuda_check(plan, cudaMemcpy(h_out, plan->d_cand, sizeof(CandRec) * n, cudaMemcpyDeviceToHost),
-                         "copy candidates")) != NSFRB_OK)
-        return st;
-    if (hdr[0] & ERR_WAIT_TIMEOUT) return fail(plan, NSFRB_ETIMEOUT, "a bulk copy into shared memory timed out");
-    if (hdr[0] & ERR_ZERO_MAD) return fail(plan, NSFRB_EINVAL, "zero MAD in at least one (pixel, subband) row");
-    if (hdr[1] > cap) return fail(plan, NSFRB_ETRUNC, "more candidates than capacity");
-    return NSFRB_OK;
+    return read_candidates(plan, h_out, cap, n_total);
 }
 
 nsfrb_status nsfrb_best(nsfrb_plan_t plan, float *out_snr, int32_t *out_idx) {
@@ -818,12 +832,12 @@ void nsfrb_destroy(nsfrb_plan_t plan) {
     if (!plan) return;
     destroy_stream_state(plan);
     if (plan->dev_ready) {
-        cudaEventSynchronize(plan->done);
-        cudaEventDestroy(plan->done);
+        cudaEventSynchronize(plan->t_end);
         cudaEventDestroy(plan->t_start);
         cudaEventDestroy(plan->t_search);
         cudaEventDestroy(plan->t_end);
     }
+    if (plan->h_res) cudaFreeHost(plan->h_res);
     cudaFree(plan->d_table);
     cudaFree(plan->d_rec);
     cudaFree(plan->d_cand);

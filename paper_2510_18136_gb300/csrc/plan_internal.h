@@ -44,8 +44,8 @@ struct nsfrb_plan_s {
     int64_t mad_slab = 0;
     float *d_full_snr = nullptr;
     int16_t *d_full_t = nullptr;
-    cudaEvent_t done = nullptr;
-    cudaEvent_t t_start = nullptr, t_search = nullptr, t_end = nullptr;   // timing of the last search
+    nsfrb::HostResult *h_res = nullptr;   // pinned, mapped; null: results are copied from the device
+    cudaEvent_t t_start = nullptr, t_search = nullptr, t_end = nullptr;   // the last search: timing, and its end
     bool searched = false;
     nsfrb_status latched = NSFRB_OK;
 
@@ -86,6 +86,7 @@ nsfrb_status queue_search(nsfrb_plan_s *pl, const void *cube, int64_t cube_pix0,
                           int t_off, const float *sigma, int64_t pix0, int64_t n, const int32_t *pix_list,
                           const int32_t *n_items_dev, int new_blk, cudaStream_t s,
                           const int32_t *t_off_dev = nullptr, int t_wrap = 0, int64_t t_stride = 0);
+nsfrb_status read_candidates(nsfrb_plan_s *pl, nsfrb_candidate *h_out, int32_t cap, int32_t *n_total);
 size_t elem_size(int dtype);
 void destroy_stream_state(nsfrb_plan_s *pl);
 void base_params(const nsfrb_plan_s *pl, SearchParams &sp);

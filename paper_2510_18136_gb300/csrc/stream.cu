@@ -251,7 +251,7 @@ nsfrb_status nsfrb_stream_open(nsfrb_plan_t plan, int32_t n_blk, size_t hbm_rese
     if (ok && qs == NSFRB_OK)
         qs = cuda_check(plan,
                         launch_compact(plan->d_rec, n_pix, c.nx, c.threshold, plan->d_counts, plan->n_blocks,
-                                       plan->d_cand, plan->d_ncand, s),
+                                       plan->d_cand, plan->d_ncand, plan->d_err, plan->h_res, s),
                         "compaction");
     cudaError_t ce = cudaStreamEndCapture(s, &graph);
     if (!ok || qs != NSFRB_OK || ce != cudaSuccess) {
@@ -339,17 +339,7 @@ nsfrb_status nsfrb_stream_poll(nsfrb_plan_t plan, int32_t timeout_ms, nsfrb_cand
     if (latency_ms &&
         (st = cuda_check(plan, cudaEventElapsedTime(latency_ms, plan->s_ev_push, plan->s_ev_done), "elapsed")))
         return st;
-    int32_t hdr[2] = {0, 0};
-    if ((st = cuda_check(plan, cudaMemcpy(hdr, plan->d_err, sizeof(hdr), cudaMemcpyDeviceToHost), "copy"))) return st;
-    *n_total = hdr[1];
-    const int32_t n = std::min(hdr[1], cap);
-    if (n > 0 && (st = cuda_check(plan, cudaMemcpy(h_out, plan->d_cand, sizeof(CandRec) * n, cudaMemcpyDeviceToHost),
-                                  "copy candidates")))
-        return st;
-    if (hdr[0] & ERR_WAIT_TIMEOUT) return fail(plan, NSFRB_ETIMEOUT, "a bulk copy into shared memory timed out");
-    if (hdr[0] & ERR_ZERO_MAD) return fail(plan, NSFRB_EINVAL, "zero MAD in at least one (pixel, subband) row");
-    if (hdr[1] > cap) return fail(plan, NSFRB_ETRUNC, "more candidates than capacity");
-    return NSFRB_OK;
+    return read_candidates(plan, h_out, cap, n_total);
 }
 
 nsfrb_status nsfrb_stream_blocks(nsfrb_plan_t plan, int64_t *n_blocks) {

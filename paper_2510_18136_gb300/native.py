@@ -236,7 +236,7 @@ class Plan:
         """``nsfrb_candidates``: structured array (row, col, dm_idx, w_idx, t_idx, snr)."""
         n = c_int32()
         cap = self.cfg.n_pix if cap is None else int(cap)
-        out = np.zeros(cap, dtype=CANDIDATE_DTYPE)
+        out = np.empty(cap, dtype=CANDIDATE_DTYPE)
         st = lib.nsfrb_candidates(self._h, out.ctypes.data_as(c_void_p), cap, ctypes.byref(n))
         _check(st, "nsfrb_candidates")
         return out[: n.value]
@@ -308,7 +308,7 @@ class Plan:
         n = c_int32()
         lat = c_float()
         cap = self.cfg.n_pix if cap is None else int(cap)
-        out = np.zeros(cap, dtype=CANDIDATE_DTYPE)
+        out = np.empty(cap, dtype=CANDIDATE_DTYPE)
         _check(lib.nsfrb_stream_poll(self._h, int(timeout_ms), out.ctypes.data_as(c_void_p), cap,
                                      ctypes.byref(n), ctypes.byref(lat)), "nsfrb_stream_poll")
         return out[: n.value], float(lat.value)
