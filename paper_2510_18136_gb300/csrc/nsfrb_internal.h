@@ -103,6 +103,7 @@ struct SearchParams {
     int32_t wide;          // 1: the wide-window kernel, mid_c samples per lane, mid_s warps per row, nb
                            // pixel buffers
     int32_t team;          // 1: the team kernel, mid_c samples per lane, teams of mid_s warps
+    int32_t serve;         // 1: the serving kernel, likewise
     // ---- outputs (indexed by absolute pixel)
     PixRec *rec;
     float *full_snr;       // [pix][n_dm][n_w] or nullptr
@@ -184,10 +185,12 @@ cudaError_t prepare_search_short(size_t smem);
 // The mid-window kernel: sets its tile, widths and shared memory in p where it applies.
 bool choose_mid(SearchParams &p, int max_smem, size_t &smem);
 cudaError_t launch_search_mid(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
-// The wide-window and team kernels, likewise.
+// The wide-window, team and serving kernels, likewise.
 bool choose_wide(SearchParams &p, int max_smem, size_t &smem);
 cudaError_t launch_search_wide(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 bool choose_team(SearchParams &p, int max_smem, size_t &smem);
+bool choose_serve(SearchParams &p, int max_smem, size_t &smem);
+cudaError_t launch_search_serve(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_search_team(const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 
 // What a search leaves in pinned, mapped host memory: its error word, the number of candidates and the

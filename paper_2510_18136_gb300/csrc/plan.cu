@@ -40,6 +40,7 @@ cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, c
     if (p.mid_w > 0) return launch_search_mid(p, grid, smem, s);
     if (p.wide) return launch_search_wide(p, grid, smem, s);
     if (p.team) return launch_search_team(p, grid, smem, s);
+    if (p.serve) return launch_search_serve(p, grid, smem, s);
     switch (C) {
         case 1: return launch_search_c1(p, grid, smem, s);
         case 3: return launch_search_c3(p, grid, smem, s);
@@ -138,6 +139,8 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
         smem = long_smem(sp, w);
         return true;
     }
+    // serving blocks of at most 32 samples: boxcars updated from row to row (figures beside the kernel)
+    if (tile_pref == 0 && choose_serve(sp, max_smem, smem)) return true;
     // windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel
     // is asked for: a lane per pixel instead of a warp per DM row.  301 x 301 pixels, FP32, against
     // the barrier-free kernel's best tile: 16 samples 71 us (1450), 32 samples 138 us (1488), 64
