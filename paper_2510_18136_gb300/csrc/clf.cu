@@ -710,11 +710,12 @@ int conv3_occupancy(int max_smem) {
 // memory fits.  The grid is the CTAs that shared memory lets reside on every SM, at most
 // 512 / (the CTA's tensor-memory columns) so that no CTA waits for tensor memory.  Returns
 // false when it does not apply (nothing launched).
-template <int CI, int CO>
+template <int CI, int CO, bool POOL = false>
 bool conv3_tc_try(const bf16 *x, const bf16 *w, float *y, float *part, int B, int D, int H, int W, int max_smem,
-                  int n_sm, int *d_err, cudaStream_t s, cudaError_t &err, int stall = 0) {
+                  int n_sm, int *d_err, cudaStream_t s, cudaError_t &err, int stall = 0,
+                  const conv3tc::PoolOut &po = conv3tc::PoolOut{}) {
     using S = conv3tc::Shape<CI, CO>;
-    if (H % conv3tc::BY || W % conv3tc::BX || W < 16 || D < 4) return false;
+    if (H % conv3tc::BY || W % conv3tc::BX || W < 16 || D < 4 || (POOL && D % 2)) return false;
     static int blocks_per_sm = 0;   // per instance: attribute set and residency computed once; -1: not usable
     if (blocks_per_sm == 0) {
         blocks_per_sm = -1;
@@ -723,10 +724,10 @@ bool conv3_tc_try(const bf16 *x, const bf16 *w, float *y, float *part, int B, in
         if (S::smem <= static_cast<size_t>(max_smem) &&
             cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess &&
-            cudaFuncSetAttribute(conv3tc::conv3_tc_kernel<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(conv3tc::conv3_tc_kernel<CI, CO, POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(S::smem)) == cudaSuccess) {
             cudaFuncAttributes fa{};
-            if (cudaFuncGetAttributes(&fa, conv3tc::conv3_tc_kernel<CI, CO>) == cudaSuccess) {
+            if (cudaFuncGetAttributes(&fa, conv3tc::conv3_tc_kernel<CI, CO, POOL>) == cudaSuccess) {
                 const int by_smem = sm_smem / static_cast<int>(S::smem + reserved);
                 const int warp_regs = (fa.numRegs * 32 + 255) / 256 * 256;   // allocation unit: 256 per warp
                 const int by_regs = 65536 / (warp_regs * (conv3tc::kThreads / 32));
@@ -738,9 +739,9 @@ bool conv3_tc_try(const bf16 *x, const bf16 *w, float *y, float *part, int B, in
     }
     if (blocks_per_sm < 1) return false;
     const int n_bricks = B * D * (H / conv3tc::BY) * (W / conv3tc::BX);
-    const int grid = std::min(n_bricks, blocks_per_sm * n_sm);
-    conv3tc::conv3_tc_kernel<CI, CO><<<grid, conv3tc::kThreads, S::smem, s>>>(x, w, y, part, D, H, W, n_bricks, d_err,
-                                                                             stall);
+    const int grid = std::min(POOL ? n_bricks / 2 : n_bricks, blocks_per_sm * n_sm);
+    conv3tc::conv3_tc_kernel<CI, CO, POOL><<<grid, conv3tc::kThreads, S::smem, s>>>(x, w, y, part, D, H, W, n_bricks,
+                                                                                   d_err, stall, po);
     err = cudaGetLastError();
     return true;
 }
@@ -824,6 +825,19 @@ bool conv3_launch(int CI, int CO, const bf16 *x, const bf16 *w, float *y, float 
     return false;
 }
 
+// Inference: convolution, batch norm, ReLU and pooling in one kernel where the tcgen05 convolution applies.
+bool conv3_pool_launch(int CI, int CO, const bf16 *x, const bf16 *w, const conv3tc::PoolOut &po, int B, int D, int H,
+                       int W, int max_smem, int n_sm, int *d_err, cudaStream_t s, cudaError_t &err) {
+    err = cudaSuccess;
+#define NSFRB_CONV3_POOL(A, Bc)                                                                              \
+    if (CI == A && CO == Bc)                                                                                 \
+        return conv3_tc_try<A, Bc, true>(x, w, nullptr, nullptr, B, D, H, W, max_smem, n_sm, d_err, s, err, 0, po);
+    NSFRB_CONV3_POOL(16, 16) NSFRB_CONV3_POOL(16, 32) NSFRB_CONV3_POOL(16, 64)
+    NSFRB_CONV3_POOL(32, 16) NSFRB_CONV3_POOL(32, 32) NSFRB_CONV3_POOL(32, 64) NSFRB_CONV3_POOL(64, 16)
+#undef NSFRB_CONV3_POOL
+    return false;
+}
+
 nsfrb_status gemm_nt(int64_t M, int N, int K, const bf16 *A, const bf16 *B, float *C, cudaStream_t s) {
     return gemm_nt_g<0>(M, N, K, A, B, C, gemm::Gather{}, s);
 }
@@ -839,8 +853,20 @@ nsfrb_status forward(nsfrb_clf_s *c, const bf16 *x, const float *labels, int B, 
     for (int l = 0; l < 4; ++l) {
         const int D = c->dims[l][0], H = c->dims[l][1], W = c->dims[l][2], Ci = c->dims[l][3], Co = cf.c[l];
         const int64_t P = static_cast<int64_t>(B) * D * H * W;
-        // training: the convolution also leaves the per-tile (128-row) channel sums of y and y^2
         cudaError_t ce;
+        if (!train) {
+            bn_eval_kernel<<<(Co + 63) / 64, 64, 0, s>>>(c->run_mean + rs, c->run_var + rs, Co, 1e-5f, c->mean[l],
+                                                         c->rstd[l]);
+            const conv3tc::PoolOut po{c->mean[l], c->rstd[l], c->params + c->off_g[l], c->params + c->off_b[l],
+                                      c->act[l + 1]};
+            if (conv3_pool_launch(Ci, Co, in, c->wb[l], po, B, D, H, W, c->max_smem, c->n_sm, clf_err(c), s, ce)) {
+                if (ce != cudaSuccess) return clf_cuda(c, ce, "conv3");
+                in = c->act[l + 1];
+                rs += Co;
+                continue;
+            }
+        }
+        // training: the convolution also leaves the per-tile (128-row) channel sums of y and y^2
         if (conv3_launch(Ci, Co, in, c->wb[l], c->y[l], train ? c->part : nullptr, B, D, H, W, c->max_smem, c->n_sm,
                          clf_err(c), s, ce)) {
             if (ce != cudaSuccess) return clf_cuda(c, ce, "conv3");
@@ -852,9 +878,6 @@ nsfrb_status forward(nsfrb_clf_s *c, const bf16 *x, const float *labels, int B, 
             const int nblk = static_cast<int>((P + kGemmRows - 1) / kGemmRows);
             bn_finish_kernel<<<Co, kFinThreads, 0, s>>>(c->part, nblk, Co, P, 1e-5f, cf.bn_momentum, 1, c->mean[l],
                                                         c->rstd[l], c->run_mean + rs, c->run_var + rs);
-        } else {
-            bn_eval_kernel<<<(Co + 63) / 64, 64, 0, s>>>(c->run_mean + rs, c->run_var + rs, Co, 1e-5f, c->mean[l],
-                                                         c->rstd[l]);
         }
         const int64_t npool = P / 8 * Co;
         bn_relu_pool_kernel<<<grid_for(npool), kTB, 0, s>>>(c->y[l], c->mean[l], c->rstd[l], c->params + c->off_g[l],
