@@ -32,6 +32,7 @@ namespace clf {
 
 using bf16 = __nv_bfloat16;
 constexpr int kTB = 256;
+constexpr int kHeadThreads = 1024;   // the head's backward (one CTA)
 
 // ------------------------------------------------------------------ Philox4x32-10
 // Salmon, Moraes, Dror, Shaw (SC 2011): ten rounds of two 32x32 multiplies
@@ -148,13 +149,30 @@ __global__ void __launch_bounds__(kTB) bn_bwd_pool_partial_kernel(const float *_
     if (ro < lanes) {
         const float mu = mean[c], rs = rstd[c], ga = gamma[c], be = beta[c];
         const int64_t w0 = static_cast<int64_t>(blockIdx.x) * wpb, w1 = min(n_win, w0 + wpb);
-        for (int64_t w = w0 + ro; w < w1; w += lanes) {
-            const int64_t i = w * C + c;
-            const int a = arg[i];
-            const float yh = (y[window_voxel(w, a, pg) * C + c] - mu) * rs;
-            const float dzv = (ga * yh + be > 0.0f) ? dpool[i] : 0.0f;
+        auto add = [&](float yv, float dp) {
+            const float yh = (yv - mu) * rs;
+            const float dzv = (ga * yh + be > 0.0f) ? dp : 0.0f;
             s += dzv;
             q += dzv * yh;
+        };
+        // four windows' loads (arg-max, then y there) in flight ahead of the adds, which keep their order
+        int64_t w = w0 + ro;
+        for (; w + 3 * lanes < w1; w += 4 * lanes) {
+            int a[4];
+            float dp[4], yv[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a[k] = arg[(w + k * lanes) * C + c];
+                dp[k] = dpool[(w + k * lanes) * C + c];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) yv[k] = y[window_voxel(w + k * lanes, a[k], pg) * C + c];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add(yv[k], dp[k]);
+        }
+        for (; w < w1; w += lanes) {
+            const int64_t i = w * C + c;
+            add(y[window_voxel(w, arg[i], pg) * C + c], dpool[i]);
         }
     }
     sh[0][threadIdx.x] = s;
@@ -318,13 +336,16 @@ __global__ void head_bwd_kernel(int B, int Fin, int F, const float *__restrict__
                                 const float *__restrict__ h1, const float *__restrict__ h1d,
                                 const float *__restrict__ logit, const float *__restrict__ labels,
                                 const float *__restrict__ w1, const float *__restrict__ w2, float p, uint2 key,
-                                uint32_t step, float *__restrict__ dh1, float *__restrict__ g_b1,
-                                float *__restrict__ g_w2, float *__restrict__ g_b2) {
-    // dh1[b][f] and the FC2 gradients (the FC1 weight gradient: head_dw1_kernel)
+                                uint32_t step, float *dh1, float *__restrict__ g_b1,
+                                float *__restrict__ g_w2, float *__restrict__ g_b2, float *dz) {
+    // dh1[b][f] and the FC2 gradients (the FC1 weight gradient: head_dw1_kernel); dz[B]
+    // (scratch) once per cutout
+    for (int b = threadIdx.x; b < B; b += blockDim.x)
+        dz[b] = (1.0f / (1.0f + expf(-logit[b])) - labels[b]) / static_cast<float>(B);
+    __syncthreads();
     for (int i = threadIdx.x; i < B * F; i += blockDim.x) {
         const int b = i / F, f = i % F;
-        const float dz = (1.0f / (1.0f + expf(-logit[b])) - labels[b]) / static_cast<float>(B);
-        float d = dz * w2[f];
+        float d = dz[b] * w2[f];
         if (p > 0.0f) {
             const uint4 u = philox4x32_10(make_uint4(static_cast<uint32_t>(b * F + f), step, 0u, 0u), key);
             const float uu = static_cast<float>(u.x >> 8) * (1.0f / 16777216.0f);
@@ -336,17 +357,17 @@ __global__ void head_bwd_kernel(int B, int Fin, int F, const float *__restrict__
     __syncthreads();
     for (int f = threadIdx.x; f < F; f += blockDim.x) {
         float sw = 0.0f, sb = 0.0f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) {
-            const float dz = (1.0f / (1.0f + expf(-logit[b])) - labels[b]) / static_cast<float>(B);
-            sw += dz * h1d[b * F + f];
+            sw += dz[b] * h1d[b * F + f];
             sb += dh1[b * F + f];
         }
         g_w2[f] = sw;
         g_b1[f] = sb;
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == blockDim.x - 1) {
         float s = 0.0f;
-        for (int b = 0; b < B; ++b) s += (1.0f / (1.0f + expf(-logit[b])) - labels[b]) / static_cast<float>(B);
+        for (int b = 0; b < B; ++b) s += dz[b];
         g_b2[0] = s;
     }
 }
@@ -359,6 +380,7 @@ __global__ void head_dw1_kernel(int B, int Fin, int F, const float *__restrict__
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int f = static_cast<int>(i / Fin), k = static_cast<int>(i - static_cast<int64_t>(f) * Fin);
         float s = 0.0f;
+#pragma unroll 8
         for (int b = 0; b < B; ++b) s += dh1[b * F + f] * feat[static_cast<int64_t>(b) * Fin + k];
         g_w1[i] = s;
     }
@@ -899,10 +921,10 @@ nsfrb_status forward(nsfrb_clf_s *c, const bf16 *x, const float *labels, int B, 
 nsfrb_status backward(nsfrb_clf_s *c, const bf16 *x, const float *labels, int B, cudaStream_t s) {
     const nsfrb_clf_config &cf = c->cfg;
     const uint2 key = make_uint2(static_cast<uint32_t>(cf.seed), static_cast<uint32_t>(cf.seed >> 32));
-    head_bwd_kernel<<<1, kTB, 0, s>>>(B, c->Fin, cf.f, c->feat, c->h1, c->h1d, c->logit, labels,
+    head_bwd_kernel<<<1, kHeadThreads, 0, s>>>(B, c->Fin, cf.f, c->feat, c->h1, c->h1d, c->logit, labels,
                                       c->params + c->off_f1w, c->params + c->off_f2w, cf.dropout, key,
                                       static_cast<uint32_t>(c->step), c->dh1, c->grads + c->off_f1b,
-                                      c->grads + c->off_f2w, c->grads + c->off_f2b);
+                                      c->grads + c->off_f2w, c->grads + c->off_f2b, c->loss_terms);
     head_dw1_kernel<<<grid_for(static_cast<int64_t>(cf.f) * c->Fin), kTB, 0, s>>>(B, c->Fin, cf.f, c->feat, c->dh1,
                                                                                 c->grads + c->off_f1w);
     head_dfeat_kernel<<<grid_for(static_cast<int64_t>(B) * c->Fin), kTB, 0, s>>>(B, c->Fin, cf.f, c->dh1,
