@@ -23,6 +23,7 @@
 //    fmaxf, so no per-element bounds test is needed.
 #pragma once
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -1191,8 +1192,17 @@ __device__ __forceinline__ void full_fill_empty(const SearchParams &p, const int
     }
 }
 
+// CTAs of 12 warps on an SM, by chunk size: a short window's row search is bound by latency, and its
+// registers leave room for more than one CTA (the barrier kernel, whose warps also wait for each other, gains
+// up to 17 samples a lane, where the barrier-free kernel's buffers leave no room).  FULL output of 9696
+// pixels, 40 DM rows, two or three CTAs against one: FP32 64 samples 357 us (750), 240 452 us (826);
+// BF16 64 412 us (1002), 240 578 us (1126), 500 1035 us (1903); FP32 MAD of 101 samples 836 us (1581).
+__host__ __device__ constexpr int ctas_per_sm(int C, bool pipe) {
+    return C <= 5 ? 3 : (C <= 9 || (C <= 17 && !pipe) ? 2 : 1);
+}
+
 template <int C, bool FULL>
-__global__ void __launch_bounds__(kThreads, 1) search_kernel(const __grid_constant__ SearchParams p) {
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(C, false)) search_kernel(const __grid_constant__ SearchParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const SmemLayout lay = smem_layout(p, C);
     int32_t *s_table = reinterpret_cast<int32_t *>(smem + lay.table);
@@ -1440,7 +1450,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel(const __grid_consta
 // of the staged row; when the copy then carries samples past the window, the de-dispersed samples
 // past the valid range are set to -inf instead of relying on -inf past the window.
 template <int C, int ST, int TEAMS, int NB, bool FULL>
-__global__ void __launch_bounds__(kThreads, 1) search_kernel_pipe(const __grid_constant__ SearchParams p) {
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(C, true)) search_kernel_pipe(const __grid_constant__ SearchParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kEs = (ST == 0) ? 4 : 2;          // bytes per stored sample
     constexpr int kEpv = 16 / kEs;                  // samples per 16 bytes
@@ -1666,6 +1676,15 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_pipe(const __grid_c
         return e;                                                                              \
     }
 
+// A persistent grid of one CTA per SM widened to the CTAs that fit (228 KB of shared memory per SM, 1 KB
+// of it per CTA).
+template <int C>
+int resident_grid(int grid, size_t smem, int64_t n_items, bool pipe) {
+    const int by_smem = std::max(1, static_cast<int>((size_t{228} << 10) / (smem + 1024)));
+    const int64_t ctas = static_cast<int64_t>(grid) * std::min(dev::ctas_per_sm(C, pipe), by_smem);
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(n_items, ctas)));
+}
+
 // The barrier kernels of a chunk size and its launch dispatch; the barrier-free kernel's launchers
 // come from NSFRB_INSTANTIATE_PIPE (16-bit ones in translation units of their own).
 #define NSFRB_INSTANTIATE_SEARCH(CC)                                                           \
@@ -1676,6 +1695,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_pipe(const __grid_c
     cudaError_t prepare_pipe_c##CC##_s1(size_t);                                               \
     cudaError_t prepare_pipe_c##CC##_s2(size_t);                                               \
     cudaError_t launch_search_c##CC(const SearchParams &p, int grid, size_t smem, cudaStream_t s) { \
+        grid = resident_grid<CC>(grid, smem, p.n_items, p.pipe != 0);                          \
         if (p.pipe) {                                                                          \
             if (p.dtype == 0) return launch_pipe_c##CC##_s0(p, grid, smem, s);                 \
             if constexpr (CC % 2 == 0) {                                                       \
