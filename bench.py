@@ -123,9 +123,10 @@ def make_cube(native, synth, cfg, seed, device, dtype):
 
 
 # DRAM bytes (read + write) per 301x301 FP32 launch from an ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum of a 128x128 launch, 1262.8 MB, scaled by 90601 / 16384 pixels), valid for the
-# kernel source with this sha256 prefix.
-NCU_TRAFFIC = {"sha256_16": "09ea857acd409e8f", "bytes": 6.981e9, "workload": (301, 301, "f32")}
+# dram__bytes_write.sum of a 128x128 launch of search_kernel_team, 1263 MB, scaled by 90601 / 16384
+# pixels), valid for the kernel source with this sha256 prefix.
+NCU_TRAFFIC = {"sha256_16": "0021d370381b00e5", "bytes": (1.26e9 + 3.22e6) * 90601 / 16384,
+               "workload": (301, 301, "f32")}
 
 
 # DRAM bytes of one imager call (grid_kernel + transform_kernel) from the ncu launch list of the
@@ -144,7 +145,7 @@ def imager_traffic():
 def measured_traffic(ny, nx, dtype):
     """ncu traffic per launch if it was taken on the current kernel source, else None."""
     import hashlib
-    src = os.path.join(ROOT, "paper_2510_18136_gb300", "csrc", "search_impl.cuh")
+    src = os.path.join(ROOT, "paper_2510_18136_gb300", "csrc", "search_team.cuh")
     with open(src, "rb") as fh:
         digest = hashlib.sha256(fh.read()).hexdigest()[:16]
     if digest != NCU_TRAFFIC["sha256_16"] or (ny, nx, dtype) != NCU_TRAFFIC["workload"]:
@@ -157,10 +158,23 @@ def search_kernel_name(n_t, dtype, noise="known", tile=None, out="candidates"):
     compiled C with 32 C > n_t.  With known noise the barrier-free kernel runs (FP32 rows; 16-bit
     rows read in place when C is even and the rows fill whole 16-byte units), with the pixel x DM
     tile (teams T, buffers per team B) the plan chose; MAD normalisation is a pass of its own into
-    FP32 slabs that the barrier-free kernel then searches.  The last template argument is FULL."""
+    FP32 slabs that the barrier-free kernel then searches.  The last template argument is FULL.
+    tile 0 (the plan kept its default): the kernels of candidate records by window length."""
     st = {"f32": 0, "bf16": 1, "f16": 2}[dtype]
     full = 1 if out == "full" else 0     # bool template arguments as ncu prints them
-    if n_t > 1247:   # beyond the register path: the long-window kernel (MAD slabs are FP32)
+    if tile == 0 and not full and n_t <= 1215:   # the default of candidate records (MAD slabs are FP32)
+        st = 0 if noise == "mad" else st
+        if n_t <= 64:
+            name = f"search_kernel_short<{next(n for n in (16, 26, 32, 48, 64) if n >= n_t)}>"
+        elif n_t <= 607:
+            tiles = ((22, 4), (26, 4), (34, 4), (22, 8), (26, 8), (34, 8), (22, 16), (26, 16), (34, 16), (38, 16))
+            name = "search_kernel_mid<%d, %d, %d>" % (*next(t for t in tiles if t[0] * t[1] > n_t), st)
+        else:
+            name = f"search_kernel_team<{next(c for c in (22, 26, 34, 38) if 32 * c > n_t)}, {st}, T, W>"
+        return f"mad_normalise_kernel + {name} (FP32 slabs)" if noise == "mad" else name
+    if n_t > 1247:   # beyond a warp's registers (MAD slabs are FP32)
+        if not full:
+            return "search_kernel_wide (search_kernel_long where a pixel does not fit in shared memory)"
         return f"search_kernel_long<{0 if noise == 'mad' else st}, {full}>"
     c = next(c for c in (1, 3, 5, 9, 17, 25, 38, 39) if 32 * c >= n_t + 1)
     tt = ", T, B" if tile is None else f", {int(tile) // 10}, {int(tile) % 10}"

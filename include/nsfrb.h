@@ -66,11 +66,12 @@ enum { NSFRB_OUT_CANDIDATES = 0, NSFRB_OUT_FULL = 1 };
 typedef struct {
     int32_t ny, nx;          /* image rows, columns (>= 1)                     */
     int32_t n_sub;           /* subbands, 1..32                                */
-    int32_t n_t;             /* window length in samples, 1..4096.  Up to 1247
-                                (the paper's 25 and 1200) a warp holds a DM
-                                row's prefix sums in registers; longer windows
-                                run a kernel that reads the cube in place and
-                                keeps the prefix sums in shared memory          */
+    int32_t n_t;             /* window length in samples, 1..4096.  Every length
+                                has a kernel of its kind: a lane per pixel (up
+                                to 64), several pixels to a warp (607), a warp
+                                per DM row (1247), several warps per DM row
+                                where a pixel fits in shared memory, and one
+                                that reads the cube in place for the rest       */
     double t_samp_ms;        /* sampling time, e.g. 134.2                      */
     double k_dm_ms;          /* dispersion constant in ms GHz^2, e.g. 4.149    */
     const double *freq_mhz;  /* [n_sub] subband centres, strictly increasing   */
@@ -175,8 +176,10 @@ nsfrb_status nsfrb_last_timing(nsfrb_plan_t plan, float *search_ms, float *total
  * search).  A tile is coded 10 * teams + buffers; NSFRB_TILES lists the
  * compiled ones.  Every tile gives the same candidates up to FP32 summation
  * order (different warps build a row group's partial sums from scratch).
- * Tile 0 = the first of 41, 31, 22, 21, 12 whose buffers fit in shared
- * memory (16-bit rows of a full window: 41; FP32 rows: 21). */
+ * Tile 0 (the default) = for candidate records of up to 1215 samples a kernel
+ * made for the window's length (n_t above) with a shape of its own; where
+ * those do not apply (FULL output, windows that are not whole 16-byte units),
+ * the first of 41, 31, 22, 21, 12 whose buffers fit in shared memory. */
 #define NSFRB_N_TILES 5
 #define NSFRB_TILES 12, 22, 21, 31, 41
 
@@ -189,9 +192,10 @@ nsfrb_status nsfrb_plan_get_tile(nsfrb_plan_t plan, int32_t dtype, int32_t *tile
 /* Time every tile that fits on the caller's cube (nsfrb_search arguments,
  * no re-score), `reps` timed searches each after one warm-up, and keep the
  * one with the smallest median search time as the plan's preference for the
- * storage type the kernel searched.  h_tile (or NULL) gets that tile (0 when
- * the plan's searches do not use this kernel: MAD windows of n_t not a
- * multiple of 4, windows over 1247 samples); h_ms[NSFRB_N_TILES] (or NULL) the medians in
+ * storage type the kernel searched.  Where tile 0 is a kernel of its own it is
+ * timed as well, and kept if it is the fastest.  h_tile (or NULL) gets the
+ * tile kept (0: that kernel, or the plan's searches have no tiles: MAD windows
+ * of n_t not a multiple of 4, windows over 1247 samples); h_ms[NSFRB_N_TILES] (or NULL) the medians in
  * NSFRB_TILES order, -1 for tiles that do not fit.  Synchronous: it waits
  * for every search it queues on `stream`.  Afterwards the plan's results are
  * those of one search of the cube with the chosen tile.  Errors: as

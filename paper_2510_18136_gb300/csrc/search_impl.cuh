@@ -1,7 +1,10 @@
 // Fused image-plane single-pulse search kernel (arXiv 2510.18136, Sec. 2.2):
 // per pixel, de-disperse every DM trial with integer shifts, boxcar-filter
 // every width with prefix sums, normalise to S/N, maximise over time, width
-// and DM.  Included by one translation unit per chunk size C.
+// and DM.  Included by one translation unit per chunk size C.  These kernels serve FULL output,
+// in-kernel MAD, rings, lists of pixels for which the kernels by window length (search_short.cu,
+// search_mid.cuh, search_team.cuh, search_wide.cuh, search_serve.cuh) do not apply, and chosen tiles;
+// the building blocks are theirs too.
 //
 // Organisation (one CTA of 12 warps per pixel, persistent over pixels):
 //  * The pixel's [n_sub][n_t] tile is staged in shared memory (bulk copies

@@ -1,5 +1,6 @@
 // The search of arXiv 2510.18136 Sec. 2.2 for windows longer than the register path holds
-// (kMaxTRegs + 1 .. kMaxT samples): per pixel and distinct DM row, the de-dispersed series
+// (kMaxTRegs + 1 .. kMaxT samples) that search_wide.cuh does not take (FULL output, rings and
+// sample-major windows, pixels that do not fit in shared memory): per pixel and distinct DM row, the de-dispersed series
 // D[t] = sum_k x_k(t + s_k), its prefix P, every width's boxcars P[t + w] - P[t] normalised by
 // 1 / (sigma sqrt(w)), and the maximum over time, width and DM with the same tie rules as the
 // other kernels (smallest DM row, then width index, then sample).
