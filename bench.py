@@ -173,7 +173,7 @@ def search_kernel_name(n_t, dtype, noise="known", tile=None, out="candidates"):
             name = f"search_kernel_team<{next(c for c in (22, 26, 34, 38) if 32 * c > n_t)}, {st}, T, W>"
         return f"mad_normalise_kernel + {name} (FP32 slabs)" if noise == "mad" else name
     if n_t > 1247:   # beyond a warp's registers (MAD slabs are FP32)
-        if not full:
+        if tile == 0 and not full:
             return "search_kernel_wide (search_kernel_long where a pixel does not fit in shared memory)"
         return f"search_kernel_long<{0 if noise == 'mad' else st}, {full}>"
     c = next(c for c in (1, 3, 5, 9, 17, 25, 38, 39) if 32 * c >= n_t + 1)
