@@ -159,7 +159,8 @@ cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, fl
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev_id);
         const int smem = kBinStages * rows * row_bytes;
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(bin_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e = cudaFuncSetAttribute(bin_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kBinStages * kBinStageBytes);   // every call's limit: see raise_smem_limit
         if (e != cudaSuccess) return e;
         int parts = 1;   // threads per output, while they and the samples last
         while (parts < 32 && 2 * parts * rows * (n_t / factor) <= kBinThreads && factor >= 16 * parts) parts *= 2;

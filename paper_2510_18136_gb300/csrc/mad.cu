@@ -459,8 +459,7 @@ template <int ST, bool VEC>
 cudaError_t launch_mad(const void *cube, int64_t pix0, int64_t n_pix, int n_sub, int n_t, float *out, uint8_t *bad,
                        int n_sm, cudaStream_t s) {
     const size_t smem = kMadWarps * warp_smem_bytes(ST == 0 ? 4 : 2, n_t);
-    cudaError_t e = cudaFuncSetAttribute(mad_normalise_kernel<ST, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(mad_normalise_kernel<ST, VEC>));
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mad_normalise_kernel<ST, VEC>, kMadWarps * 32, smem);

@@ -169,6 +169,11 @@ inline int pick_chunk(int n_t) {
     return n_t <= kMaxT ? kLongC : -1;
 }
 
+// Raises a kernel's limit of dynamic shared memory to what the device allows beside static_bytes of its own.
+// The limit belongs to the function, not to a plan, stream or thread, so it is never set to the need of
+// one launch: another plan would lower it between a larger plan's call here and its launch.
+cudaError_t raise_smem_limit(const void *kernel, int static_bytes = 0);
+
 // Kernel launchers (one translation unit per chunk size; C = kLongC: the long-window kernel).
 cudaError_t launch_search(int C, const SearchParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t prepare_search(int C, size_t smem);

@@ -74,6 +74,14 @@ cudaError_t prepare_search(int C, size_t smem) {
     }
 }
 
+cudaError_t raise_smem_limit(const void *kernel, int static_bytes) {
+    int dev = 0, limit = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit - static_bytes);
+}
+
 size_t elem_size(int dtype) { return dtype == NSFRB_F32 ? 4 : 2; }
 
 // Fill the parts of SearchParams that depend only on the plan.

@@ -372,8 +372,7 @@ cudaError_t mid_launch(const SearchParams &p, int grid_sm, size_t smem, cudaStre
     // where only the device knows the count, as many CTAs as can run at once (at most) loop over it
     const int64_t sets = (p.n_items + 32 / S - 1) / (32 / S);
     const unsigned grid = static_cast<unsigned>(p.n_items_dev ? std::min<int64_t>(sets, 2 * grid_sm) : sets);
-    const cudaError_t e = cudaFuncSetAttribute(search_kernel_mid<C, S, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(search_kernel_mid<C, S, ST>));
     if (e != cudaSuccess) return e;
     search_kernel_mid<C, S, ST><<<grid, 32 * p.mid_w, smem, s>>>(p);
     return cudaGetLastError();

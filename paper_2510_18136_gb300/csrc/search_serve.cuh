@@ -295,8 +295,7 @@ __global__ void __launch_bounds__(TEAMS * W * 32, 1) search_kernel_serve(const _
 
 template <int C, int ST, int TEAMS, int W>
 cudaError_t serve_launch(const SearchParams &p, int n_sm, size_t smem, cudaStream_t s) {
-    const cudaError_t e = cudaFuncSetAttribute(search_kernel_serve<C, ST, TEAMS, W>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(search_kernel_serve<C, ST, TEAMS, W>));
     if (e != cudaSuccess) return e;
     search_kernel_serve<C, ST, TEAMS, W><<<n_sm, TEAMS * W * 32, smem, s>>>(p);
     return cudaGetLastError();

@@ -381,8 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_wide(const __grid_c
 
 template <int C, int V, int ST>
 cudaError_t wide_launch(const SearchParams &p, int grid, size_t smem, cudaStream_t s) {
-    const cudaError_t e = cudaFuncSetAttribute(search_kernel_wide<C, V, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(search_kernel_wide<C, V, ST>));
     if (e != cudaSuccess) return e;
     search_kernel_wide<C, V, ST><<<grid, kThreads, smem, s>>>(p);
     return cudaGetLastError();
