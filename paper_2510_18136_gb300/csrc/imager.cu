@@ -605,10 +605,9 @@ nsfrb_status nsfrb_imager_create(const nsfrb_imager_config *cfg, nsfrb_imager_t 
         (st = up(reinterpret_cast<void **>(&im->d_tab), tab.data(), sizeof(float) * tab.size())) ||
         (st = cuda_check(nullptr, cudaMalloc(&im->d_err, sizeof(int32_t)), "cudaMalloc")) ||
         (st = cuda_check(nullptr, cudaMemset(im->d_err, 0, sizeof(int32_t)), "memset")) ||
-        (st = cuda_check(nullptr, cudaFuncSetAttribute(grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      static_cast<int>(im->gs.total)), "smem attribute")) ||
-        (st = cuda_check(nullptr, cudaFuncSetAttribute(transform_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      static_cast<int>(im->tr.total)), "smem attribute"))) {
+        (st = cuda_check(nullptr, raise_smem_limit(reinterpret_cast<const void *>(grid_kernel), 1024), "smem attribute")) ||
+        (st = cuda_check(nullptr, raise_smem_limit(reinterpret_cast<const void *>(transform_kernel)),
+                         "smem attribute"))) {
         if (st == NSFRB_ECUDA && std::string(nsfrb_last_error()).find("out of memory") != std::string::npos)
             st = NSFRB_ENOMEM;
         imager_free(im);

@@ -94,3 +94,23 @@ def test_serving_of_two_open_streams(native):
             assert len(cand) == 0
     for plan, _ in plans:
         plan.close()
+
+
+def test_two_imagers(native):
+    """An imager of a smaller uv support made after a larger one; the larger one still images, same bits."""
+    from paper_2510_18136_gb300 import synth_vis
+
+    def make(n_ew, n_ns, n_grid):
+        uv = synth_vis.baseline_uv(synth_vis.core_layout(0, n_ew, n_ns))
+        chan = synth_vis.channel_freqs(4, 2)
+        vis = synth_vis.visibilities(uv, chan, 1, [(3, -5, np.ones((1, 4)))], noise=1.0, seed=1, device="cuda")
+        return native.Imager(uv, chan, n_grid=n_grid), vis
+
+    large, vis = make(48, 34, 175)
+    before = large.image(vis).clone()
+    small, vis_small = make(12, 8, 64)
+    small.image(vis_small)
+    assert torch.equal(large.image(vis), before)
+    large.status()
+    small.close()
+    large.close()
