@@ -102,6 +102,7 @@ struct SearchParams {
                                    // lanes per pixel
     int32_t wide;          // 1: the wide-window kernel, mid_c samples per lane, mid_s warps per row, nb
                            // pixel buffers
+    int32_t wide_lo;       // 1: and the rounding errors of the chunks' prefixes
     int32_t team;          // 1: the team kernel, mid_c samples per lane, teams of mid_s warps
     int32_t serve;         // 1: the serving kernel, likewise
     // ---- outputs (indexed by absolute pixel)

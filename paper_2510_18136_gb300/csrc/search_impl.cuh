@@ -636,6 +636,80 @@ __device__ __forceinline__ float small_max_pk(const float2 (&D)[C / 2], const fl
     return fmax3(acc[0], acc[1], acc[2]);
 }
 
+// The next lane's first 15 samples, which boxcars of up to 16 samples that start in this chunk reach.  The last
+// lane needs no mask: its chunk's last sample is past the window (-inf or NaN), and every boxcar that
+// leaves the chunk holds it.
+template <int C>
+__device__ __forceinline__ void halo_samples(const float2 (&D)[C / 2], float2 (&Hd)[kSmallMax / 2]) {
+#pragma unroll
+    for (int i = 0; i + 1 < kSmallMax; ++i) pset(Hd, i, __shfl_down_sync(kFull, pget(D, i), 1));
+    Hd[kSmallMax / 2 - 1].y = 0.0f;
+}
+
+// Maxima of the in-lane boxcars of 1, 2, 4, 8 and 16 samples (each(J, maximum) for J = 0 .. top) by doubling,
+// B2[t] = D[t] + D[t + 1], B4[t] = B2[t] + B2[t + 2], ..., from the chunk and the 15 samples after it (Hd): without a
+// prefix, so that a bright or invalid sample outside a boxcar leaves nothing in it.  Returns the
+// maximum of the 32-sample boxcars that lie within the chunk (-inf where C <= 32 or top < 4).
+template <int C, typename F>
+__device__ __forceinline__ float small_sums(const float2 (&D)[C / 2], const float2 (&Hd)[kSmallMax / 2], int top, F each) {
+    static_assert(C % 2 == 0 && kSmallMax == 16, "pairs; 15 samples of halo");
+    constexpr int N = (C + 16) / 2;
+    float2 E[N];
+    auto best = [&]() {
+        float acc[3] = {neg_inf(), neg_inf(), neg_inf()};
+#pragma unroll
+        for (int m = 0; m < C / 2; ++m) acc[m % 3] = fmax3(acc[m % 3], E[m].x, E[m].y);
+        return fmax3(acc[0], acc[1], acc[2]);
+    };
+#pragma unroll
+    for (int m = 0; m < N; ++m) E[m] = m < C / 2 ? D[m] : Hd[m - C / 2];
+    each(0, best());
+    if (top < 1) return neg_inf();
+#pragma unroll
+    for (int i = 0; i < C + 14; ++i) pset(E, i, pget(E, i) + pget(E, i + 1));
+    each(1, best());
+    if (top < 2) return neg_inf();
+#pragma unroll
+    for (int m = 0; m < (C + 12) / 2; ++m) E[m] = add2(E[m], E[m + 1]);
+    each(2, best());
+    if (top < 3) return neg_inf();
+#pragma unroll
+    for (int m = 0; m < (C + 8) / 2; ++m) E[m] = add2(E[m], E[m + 2]);
+    each(3, best());
+    if (top < 4) return neg_inf();
+#pragma unroll
+    for (int m = 0; m < C / 2; ++m) E[m] = add2(E[m], E[m + 4]);
+    each(4, best());
+    float m32 = neg_inf();
+    if constexpr (C > 32) {
+#pragma unroll
+        for (int m = 0; m < (C - 32) / 2; ++m) {
+            const float2 b = add2(E[m], E[m + 8]);
+            m32 = fmax3(m32, b.x, b.y);
+        }
+    }
+    return m32;
+}
+
+// The largest J <= 4 with a width of 1 << J among the plan's (J = 4 where 32 samples may lie within a chunk).
+template <int C>
+__device__ __forceinline__ int small_top(const SearchParams &p) {
+    if (C > 32 && p.pow2_wi[5] >= 0) return 4;
+    int top = 0;
+#pragma unroll
+    for (int j = 1; j < 5; ++j)
+        if (p.pow2_wi[j] >= 0) top = j;
+    return top;
+}
+
+// (h, l) += (bh, bl): sums kept as an FP32 value and its rounding error (two-sum), so that a difference of two
+// of them has the error of the difference itself.
+__device__ __forceinline__ void pair_add(float &h, float &l, float bh, float bl) {
+    const float s = h + bh, bb = s - h;
+    l += ((h - (s - bb)) + (bh - bb)) + bl;
+    h = s;
+}
+
 // Lane-strided P as pairs: Ps[m] = (P[64 m + lane], P[64 m + 32 + lane]).
 template <int C>
 __device__ __forceinline__ void load_ps(const float *Pw, int lane, float2 (&Ps)[C / 2]) {

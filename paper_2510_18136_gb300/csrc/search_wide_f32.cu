@@ -23,6 +23,22 @@ bool choose_wide(SearchParams &p, int max_smem, size_t &smem) {
     NSFRB_WIDE_TILES(NSFRB_WIDE_PICK)
 #undef NSFRB_WIDE_PICK
     if (C == 0) return false;
+    // power-of-two widths have their own code; the others, where shorter than a chunk, need the rounding
+    // errors of the chunks' prefixes
+    p.n_gen = p.has_large = p.wide_lo = 0;
+    for (int j = 0; j < kPow2; ++j) p.pow2_wi[j] = -1;
+    for (int i = 0; i < p.n_w; ++i) {
+        int j = -1;
+        for (int b = 0; b < kPow2; ++b)
+            if (p.widths[i] == (1 << b)) j = b;
+        if (j >= 0) {
+            p.pow2_wi[j] = i;
+            p.has_large |= p.widths[i] > kSmallMax;
+        } else {
+            p.gen_wi[p.n_gen++] = i;
+            p.wide_lo |= p.widths[i] < C;
+        }
+    }
     int nb = 2;
     while (nb > 0 && dev::wide_layout(p, C, V, nb).total > static_cast<size_t>(max_smem)) --nb;
     if (nb == 0) return false;
@@ -33,20 +49,6 @@ bool choose_wide(SearchParams &p, int max_smem, size_t &smem) {
     p.wide = 1;
     p.nb = nb;
     smem = dev::wide_layout(p, C, V, nb).total;
-    // power-of-two widths have their own code where a chunk and the one after it span them
-    p.n_gen = p.has_large = 0;
-    for (int j = 0; j < kPow2; ++j) p.pow2_wi[j] = -1;
-    for (int i = 0; i < p.n_w; ++i) {
-        int j = -1;
-        for (int b = 0; b < kPow2; ++b)
-            if (p.widths[i] == (1 << b) && (1 << b) < 64 * C) j = b;
-        if (j >= 0) {
-            p.pow2_wi[j] = i;
-            p.has_large |= p.widths[i] > kSmallMax;
-        } else {
-            p.gen_wi[p.n_gen++] = i;
-        }
-    }
     return true;
 }
 
