@@ -4,8 +4,10 @@
 // A warp per DM row of such a window leaves a lane 3 to 19 samples, and the row costs what its
 // dependent chain costs (warp scan, shared-memory round trip, warp maxima), whatever its length.
 // Here a warp searches the same DM row of 32 / S pixels at once, S lanes to a pixel, and a lane owns a
-// chunk of C samples as long as the full window's kernel gives it, with the same per-lane code:
-// sample pairs, in-lane prefix and halo, P to shared memory, lane-strided widths from there.
+// chunk of C samples as long as the full window's kernel gives it: sample pairs, widths up to 16 by doubling
+// in registers (small_sums: the kernels before had chunks of 3 to 17 samples, and an in-lane prefix over 22
+// to 38 would put a bright or invalid sample into more of them), P to shared memory, lane-strided
+// widths from there.
 //  * A CTA takes 32 / S consecutive pixels, its warps contiguous groups of the distinct DM rows.  A
 //    pixel's rows lie packed in shared memory as stored (16-bit rows read in place), one
 //    bulk copy per pixel.  The pixel pitch is C S modulo 32 words: the lanes' chunks then go on from
@@ -17,13 +19,14 @@
 //    P[t + w] is a register of the same lane for every power of two w >= 2 S.
 //  * Each lane tracks its own best (S/N, row, width) over all rows: no warp maxima per row.  At the end
 //    a warp per pixel rebuilds the best row from all subbands, and takes the record's S/N and the
-//    earliest sample reaching it from that row.
+//    earliest sample reaching it from that row, with the same two forms of boxcars.
 // Bound by instruction issue and, for few rows, by the copies (two or three CTAs fit on an SM, so
 // copy and search overlap only between them).  C and S are the smallest of the compiled windows S C
 // that hold the samples; the rows are split over as many warps as keep the SM's register file full.
 // 301 x 301 pixels x 16 subbands, 40 distinct DM rows, power-of-two widths, against the kernels
-// with a warp per row: FP32 100 samples 503 us (2873), 240 1284 us (2947), 400 2111 us (3261), 600
-// 2940 us (4409); BF16 240 1079 us (4887), 300 1494 us (9300), 600 2515 us (7077).
+// with a warp per row: FP32 100 samples 533 us (2873), 240 1311 us (2947), 400 2208 us (3261), 600
+// 2986 us (4409); BF16 240 1114 us (4887), 300 1567 us (9300), 600 2580 us (7077).  With in-lane prefixes
+// for the widths up to 16: 521, 1295, 2178, 3001; 1098, 1540, 2561 us.
 #pragma once
 
 #include <algorithm>
@@ -93,7 +96,7 @@ template <int C, int S, int ST>
 __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const __grid_constant__ SearchParams p) {
     static_assert(C % 4 == 2 && C >= kSmallMax, "pairs without bank conflicts; the halo is one chunk at most");
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr int PW = 32 / S, SH = kSmallMax, kEs = (ST == 0) ? 4 : 2;
+    constexpr int PW = 32 / S, kEs = (ST == 0) ? 4 : 2;
     const int n_warps = blockDim.x >> 5;
     const MidLayout lay = mid_layout(p, C, S, n_warps);
     int32_t *s_table = reinterpret_cast<int32_t *>(smem + lay.table);
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
+    const int top = small_top<26>(p);   // (32 samples are lane-strided here, whatever the chunk)
     uint32_t phase = 0;
     // one set of pixels per CTA, or, where a device count says how many there are (re-scoring), several
     for (int64_t it0 = static_cast<int64_t>(blockIdx.x) * PW; it0 < n_items;
@@ -214,11 +218,15 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                 }
             };
             {
-                float2 Lp[C / 2], Hh[SH / 2];
+                float2 Hd[kSmallMax / 2];
+                halo_samples<C>(D, Hd);   // a pixel's last lane takes the next pixel's: see there
+                small_sums<C>(D, Hd, top, [&](int b, float m) {
+                    if (p.pow2_wi[b] >= 0) consider(p.pow2_wi[b], m);
+                });
+            }
+            {
+                float2 Lp[C / 2];
                 const float tot = prefix_pairs<C>(D, Lp);
-                // the last chunk of a pixel ends past its window: its total is -inf or NaN, and with it
-                // the halo that its last lane takes from the next pixel's first
-                halo_pairs<C, SH>(Lp, tot, Hh);
                 float inc = tot;
 #pragma unroll
                 for (int o = 1; o < S; o <<= 1) {
@@ -227,10 +235,6 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                 }
                 float carry = __shfl_up_sync(kFull, inc, 1, S);
                 if (j == 0) carry = 0.0f;
-#define NSFRB_MID_SMALL(J) \
-    if (p.pow2_wi[J] >= 0) consider(p.pow2_wi[J], small_max_pk<C, SH, (1 << J)>(D, Lp, Hh));
-                NSFRB_MID_SMALL(0) NSFRB_MID_SMALL(1) NSFRB_MID_SMALL(2) NSFRB_MID_SMALL(3) NSFRB_MID_SMALL(4)
-#undef NSFRB_MID_SMALL
                 store_p<C>(Pw, lane * C, carry, Lp);
             }
             __syncwarp();
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
 #pragma unroll
                 for (int m = 0; m < C / 2; ++m) Ps[m] = src2[S * m];
 #define NSFRB_MID_LARGE(J)                                                                     \
-    if constexpr ((1 << J) > SH && (1 << J) < S * C) {                                         \
+    if constexpr ((1 << J) > kSmallMax && (1 << J) < S * C) {                                         \
         if (p.pow2_wi[J] >= 0) consider(p.pow2_wi[J], mid_large<C, (1 << J) / (2 * S)>(Ps));  \
     }
                 NSFRB_POW2(NSFRB_MID_LARGE)
@@ -311,9 +315,11 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                         }
                     }
                 }
-                // w = 1: D in the buffer; else P, with P[t1 + c] kept in d[c]
+                // widths of the in-lane path: the samples in the buffer, boxcars by doubling as in small_sums;
+                // others: P in the buffer, with P[t1 + c] kept in d[c]
+                const bool small = w <= kSmallMax && (w & (w - 1)) == 0;
                 __syncwarp();
-                if (w == 1) {
+                if (small) {
 #pragma unroll
                     for (int c = 0; c < CC; ++c)
                         if (t1 + c < L) Pw[t1 + c] = d[c];
@@ -333,11 +339,25 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                     }
                 }
                 __syncwarp();
+                if (small) {
+                    constexpr int N = CC + kSmallMax - 1;
+                    float x[N];
+#pragma unroll
+                    for (int c = 0; c < N; ++c) x[c] = c < CC ? d[c] : (c < CC + w - 1 && t1 + c < L) ? Pw[t1 + c] : 0.0f;
+#pragma unroll
+                    for (int h = 1; h < kSmallMax; h *= 2) {
+                        if (w <= h) break;
+#pragma unroll
+                        for (int c = 0; c + h < N; ++c) x[c] += x[c + h];
+                    }
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) d[c] = x[c];
+                }
                 float m = neg_inf();
 #pragma unroll
                 for (int c = 0; c < CC; ++c) {
                     if (t1 + c + w <= L) {
-                        if (w > 1) d[c] = Pw[t1 + c + w] - d[c];
+                        if (!small) d[c] = Pw[t1 + c + w] - d[c];
                         m = fmaxf(m, d[c]);
                     }
                 }

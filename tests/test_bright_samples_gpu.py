@@ -3,7 +3,8 @@
 A dirty image has deep negative sidelobes and, where data were flagged, samples that are not numbers.  The
 record of a pixel is compared with the best trial that holds no such sample:
 
-* S/N within parity's 1e-5.  A boxcar of the wide kernel is summed from its own samples, so its error is a few times 2^-24 of its own value whatever
+* S/N within parity's 1e-5.  A boxcar of the wide kernel and of the in-lane widths of the mid kernel
+  is summed from its own samples, so its error is a few times 2^-24 of its own value whatever
   lies outside it; sums that ran over a sample of -1e4 would be off by 2^-24 x 1e4 = 6e-4, 1e-5
   to 4e-5 of an S/N of 4 to 14 at the widths used.
 * the indices wherever the margin to the next trial is clear.
@@ -43,11 +44,13 @@ def _search(native, cfg, cube, sig, dtype):
 
 
 # every width where no long prefix is differenced (wide; not 3 and 25 with 2400 FP32 samples, which the long-window
-# kernel takes)
+# kernel takes), the in-lane widths elsewhere
 ALL = [1, 2, 3, 4, 8, 16, 25, 32, 64, 100, 128, 256, 512, 1024, 1200]
 
 
 @pytest.mark.parametrize("n_t,dtype,widths", [
+    (80, "f32", [1, 2, 4, 8, 16]), (95, "bf16", [1, 2, 4, 8, 16]), (240, "f32", [1, 2, 4, 8, 16]),
+    (287, "f16", [1, 4, 16]), (400, "bf16", [2, 8, 16]), (600, "f32", [1, 2, 4, 8, 16]),
     (1250, "f32", ALL), (1407, "bf16", ALL), (1664, "f32", ALL), (2048, "f32", ALL), (2048, "bf16", ALL + [2048]),
     (2175, "bf16", ALL), (2400, "f32", [v for v in ALL if v not in (3, 25)]), (3000, "bf16", ALL), (4096, "f16", ALL),
 ])
@@ -76,7 +79,8 @@ def _direct(x, sh, w, t):
 
 
 @pytest.mark.parametrize("value", [float("nan"), float("-inf")])
-@pytest.mark.parametrize("n_t,dtype,w", [(1250, "f32", 4),
+@pytest.mark.parametrize("n_t,dtype,w", [(80, "f32", 4), (240, "bf16", 4), (240, "f32", 8),
+                                         (600, "f32", 16), (700, "f32", 8), (1200, "bf16", 16), (1250, "f32", 4),
                                          (2048, "f32", 16), (2048, "bf16", 2), (2048, "f32", 3), (4000, "bf16", 8)])
 def test_pulse_after_an_invalid_sample(native, n_t, dtype, w, value):
     """A strong pulse of an in-lane width after (or before) an invalid sample is the record."""
