@@ -10,7 +10,8 @@
 //    for all lanes.
 //  * A thread holds its pixel's de-dispersed row D[t] and prefix P[t] in registers and updates D from one
 //    row to the next by the subbands whose shift changed, as the other kernels do.  Prefix,
-//    boxcars and maxima need no communication between lanes.
+//    boxcars and maxima need no communication between lanes.  Pairs of samples (w = 2) are summed
+//    without the prefix: a sample that is not a number, or a bright one, does not reach those after it.
 //  * D past the valid range is set to -inf; later rows of a group have shorter ranges (delays
 //    grow with the DM), so an element once out of range stays out, and every trial that reads
 //    it is -inf or NaN and drops out of the maximum.
@@ -59,13 +60,18 @@ __host__ __device__ inline ShortLayout short_layout(const SearchParams &p, int n
     return L;
 }
 
-// Maximum over t of the boxcars of width W: D itself for W = 1, else P[t + W] - P[t].
+// Maximum over t of the boxcars of width W: D itself for W = 1, D[t] + D[t + 1] for W = 2, else P[t + W] - P[t].
 template <int NT, int W>
 __device__ __forceinline__ float short_max(const float2 (&D)[NT / 2], const float2 (&P)[NT / 2 + 1]) {
     float acc[3] = {neg_inf(), neg_inf(), neg_inf()};
     if constexpr (W == 1) {
 #pragma unroll
         for (int m = 0; m < NT / 2; ++m) acc[m % 3] = fmax3(acc[m % 3], D[m].x, D[m].y);
+    } else if constexpr (W == 2) {
+#pragma unroll
+        for (int t = 0; t + 2 < NT; t += 2)
+            acc[(t >> 1) % 3] = fmax3(acc[(t >> 1) % 3], pget(D, t) + pget(D, t + 1), pget(D, t + 1) + pget(D, t + 2));
+        acc[2] = fmaxf(acc[2], pget(D, NT - 2) + pget(D, NT - 1));
     } else if constexpr (W % 2 == 0) {
         constexpr int N = NT - W + 1;   // trials t = 0 .. NT - W
 #pragma unroll
@@ -281,8 +287,8 @@ search_kernel_short(const __grid_constant__ SearchParams p) {
             if (any) {
                 const int w = p.widths[bwi];
                 const float inv = s_inv[bwi * kShortPix + lane];
-                float *col = xs + lane;   // D[t] at col[t * 32]; P[t] in its place for w > 1
-                if (w > 1) {
+                float *col = xs + lane;   // D[t] at col[t * 32]; P[t] in its place for w > 2
+                if (w > 2) {
                     float run = 0.0f;
                     for (int t = 0; t <= L; ++t) {
                         const float v = t < L ? col[t * kShortPix] : 0.0f;
@@ -290,7 +296,13 @@ search_kernel_short(const __grid_constant__ SearchParams p) {
                         run += v;
                     }
                 }
-                auto box = [&](int t) { return w == 1 ? col[t * kShortPix] : col[(t + w) * kShortPix] - col[t * kShortPix]; };
+                // boxcar t = b[t] + ca a[t] (exact product): D[t] + 0 for w = 1, D[t + 1] + D[t], P[t + w] - P[t]; lanes
+                // differ in w, so no branches
+                const float *b = col + (w == 1 ? 0 : w == 2 ? 1 : w) * kShortPix;
+                const float *a = w == 1 ? xs + (size_t)kShortPix * pitch + kShortPad - 1 : col;
+                const int sa = w == 1 ? 0 : kShortPix;
+                const float ca = w <= 2 ? 1.0f : -1.0f;
+                auto box = [&](int t) { return fmaf(ca, a[t * sa], b[t * kShortPix]); };
                 float m = neg_inf();
                 for (int t = 0; t + w <= L; ++t) m = fmaxf(m, box(t));
                 r.snr = m * inv;

@@ -3,8 +3,8 @@
 A dirty image has deep negative sidelobes and, where data were flagged, samples that are not numbers.  The
 record of a pixel is compared with the best trial that holds no such sample:
 
-* S/N within parity's 1e-5.  A boxcar of the wide kernel and of the in-lane widths of the mid kernel
-  is summed from its own samples, so its error is a few times 2^-24 of its own value whatever
+* S/N within parity's 1e-5.  A boxcar of the wide kernel and of the in-lane widths of the mid and short
+  kernels is summed from its own samples, so its error is a few times 2^-24 of its own value whatever
   lies outside it; sums that ran over a sample of -1e4 would be off by 2^-24 x 1e4 = 6e-4, 1e-5
   to 4e-5 of an S/N of 4 to 14 at the widths used.
 * the indices wherever the margin to the next trial is clear.
@@ -49,6 +49,7 @@ ALL = [1, 2, 3, 4, 8, 16, 25, 32, 64, 100, 128, 256, 512, 1024, 1200]
 
 
 @pytest.mark.parametrize("n_t,dtype,widths", [
+    (50, "f32", [1, 2]), (50, "bf16", [1, 2]), (64, "f32", [1, 2]),
     (80, "f32", [1, 2, 4, 8, 16]), (95, "bf16", [1, 2, 4, 8, 16]), (240, "f32", [1, 2, 4, 8, 16]),
     (287, "f16", [1, 4, 16]), (400, "bf16", [2, 8, 16]), (600, "f32", [1, 2, 4, 8, 16]),
     (1250, "f32", ALL), (1407, "bf16", ALL), (1664, "f32", ALL), (2048, "f32", ALL), (2048, "bf16", ALL + [2048]),
@@ -79,7 +80,7 @@ def _direct(x, sh, w, t):
 
 
 @pytest.mark.parametrize("value", [float("nan"), float("-inf")])
-@pytest.mark.parametrize("n_t,dtype,w", [(80, "f32", 4), (240, "bf16", 4), (240, "f32", 8),
+@pytest.mark.parametrize("n_t,dtype,w", [(60, "f32", 2), (60, "bf16", 1), (80, "f32", 4), (240, "bf16", 4), (240, "f32", 8),
                                          (600, "f32", 16), (700, "f32", 8), (1200, "bf16", 16), (1250, "f32", 4),
                                          (2048, "f32", 16), (2048, "bf16", 2), (2048, "f32", 3), (4000, "bf16", 8)])
 def test_pulse_after_an_invalid_sample(native, n_t, dtype, w, value):
