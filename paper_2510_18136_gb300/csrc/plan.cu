@@ -785,26 +785,34 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
     if (!plan || !d_cube || reps < 1) return fail(plan, NSFRB_EINVAL, "bad argument");
     if (h_ms)
         for (int k = 0; k < NSFRB_N_TILES; ++k) h_ms[k] = -1.0f;
-    // one untimed search finds the storage type the barrier-free kernel would search (the slabs of
-    // MAD mode are FP32) or that it does not apply
+    // one untimed search with the default (tile 0), whatever tile the plan holds, finds the storage type that is
+    // searched (the slabs of MAD mode are FP32), whether it has tiles, and whether the default is a kernel of its own
+    int32_t keep[3];
+    std::memcpy(keep, plan->tile, sizeof(keep));
+    std::memset(plan->tile, 0, sizeof(keep));
+    auto restore = [&]() { std::memcpy(plan->tile, keep, sizeof(keep)); };
     nsfrb_status st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
     if (st == NSFRB_OK) st = nsfrb_last_timing(plan, nullptr, nullptr);
-    if (st != NSFRB_OK) return st;
     const int s_t = plan->last_tile_st;
+    restore();
+    if (st != NSFRB_OK) return st;
     if ((plan->last_tile == 0 && !plan->last_other) || s_t < 0) {
         if (h_tile) *h_tile = 0;
         return NSFRB_OK;
     }
-    const int32_t keep = plan->tile[s_t];
     int32_t best = 0;
     float best_ms = 0.0f;
     bool timed = false;   // best_ms holds a time
     std::vector<float> t(reps);
     if (plan->last_other) {   // tile 0 is another kernel: a contender of its own
+        plan->tile[s_t] = 0;
         for (int r = 0; r < reps; ++r) {
             st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
             if (st == NSFRB_OK) st = nsfrb_last_timing(plan, &t[r], nullptr);
-            if (st != NSFRB_OK) return st;
+            if (st != NSFRB_OK) {
+                restore();
+                return st;
+            }
         }
         std::sort(t.begin(), t.end());
         best_ms = t[reps / 2];
@@ -816,7 +824,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
             st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
             if (st == NSFRB_OK) st = nsfrb_last_timing(plan, r >= 0 ? &t[r] : nullptr, nullptr);
             if (st != NSFRB_OK) {
-                plan->tile[s_t] = keep;
+                restore();
                 return st;
             }
             if (plan->last_tile != kTileCodes[k]) break;   // does not fit: another tile ran
@@ -831,7 +839,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
             timed = true;
         }
     }
-    plan->tile[s_t] = timed ? best : keep;
+    plan->tile[s_t] = timed ? best : keep[s_t];
     if (h_tile) *h_tile = plan->tile[s_t];
     // the plan's results are those of a search with the chosen tile
     st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);

@@ -88,3 +88,19 @@ def test_short_window_autotune_keeps_results(native):
     for k in ("row", "col", "dm_idx", "w_idx", "t_idx"):
         assert (before[k] == after[k]).all()
     assert np.abs(before["snr"] - after["snr"]).max() <= 1e-5 * before["snr"].max()
+
+
+def test_autotune_times_the_default_of_a_plan_with_a_tile(native):
+    """A plan that holds a tile: autotune still times tile 0 (a lane per pixel, twice as fast here) and keeps it."""
+    cfg = synth.SearchConfig(ny=64, nx=64, n_t=24, dm=np.linspace(0.0, 2000.0, 16),
+                             widths=np.array([1, 2, 4, 8, 16], np.int32), threshold=9.0)
+    cube = synth.plain_noise(cfg, 1).cuda()
+    with native.Plan(cfg) as plan:
+        plan.set_tile(native.F32, 41)
+        tile, ms = plan.autotune(cube, reps=5)
+        assert tile == 0 and plan.get_tile(native.F32) == 0
+        assert 41 in ms
+        # a storage type that was not searched keeps its tile
+        plan.set_tile(native.BF16, 22)
+        plan.autotune(cube, reps=1)
+        assert plan.get_tile(native.BF16) == 22
