@@ -198,7 +198,9 @@ nsfrb_status nsfrb_plan_get_tile(nsfrb_plan_t plan, int32_t dtype, int32_t *tile
  * of n_t not a multiple of 4, windows over 1247 samples); h_ms[NSFRB_N_TILES] (or NULL) the medians in
  * NSFRB_TILES order, -1 for tiles that do not fit.  Synchronous: it waits
  * for every search it queues on `stream`.  Afterwards the plan's results are
- * those of one search of the cube with the chosen tile.  Errors: as
+ * those of one search of the cube with the chosen tile.  Blocks of a stream
+ * keep their own kernel beside a tile kept here (not beside one set by
+ * nsfrb_plan_set_tile).  Errors: as
  * nsfrb_search; EINVAL for reps < 1. */
 nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const float *d_sigma, int32_t reps,
                                  void *stream, int32_t *h_tile, float *h_ms);

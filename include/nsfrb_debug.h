@@ -54,6 +54,15 @@ nsfrb_status nsfrb_dbg_wait_timeout(int32_t limit_ms);
 nsfrb_status nsfrb_dbg_mad_normalise(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, float *d_out,
                                      uint8_t *d_bad, void *stream);
 
+/* The kernel that a search of n_items of the plan's pixels would run on a device with 227 KB of
+ * shared memory per block, for rows stored as dtype at an address `offset` bytes past a multiple of
+ * 16; new_blk > 0: a block of that many samples of a served window.  tile, tuned: the tile
+ * that the plan would hold, and whether autotune kept it.  Host code only.  Returns 1 the
+ * barrier kernel, 2 the barrier-free kernel, 3 the long-window kernel, 4 short, 5 mid, 6 wide,
+ * 7 team, 8 serving; 0 where nothing fits, -1 for bad arguments. */
+int32_t nsfrb_dbg_search_kernel(nsfrb_plan_t plan, int32_t dtype, int64_t n_items, int32_t offset, int32_t new_blk,
+                                int32_t tile, int32_t tuned);
+
 #ifdef __cplusplus
 }
 #endif

@@ -42,6 +42,38 @@ extern "C" nsfrb_status nsfrb_dbg_wait_timeout(int32_t limit_ms) {
     return (h_err & ERR_WAIT_TIMEOUT) ? NSFRB_ETIMEOUT : NSFRB_OK;
 }
 
+extern "C" int32_t nsfrb_dbg_search_kernel(nsfrb_plan_t plan, int32_t dtype, int64_t n_items, int32_t offset,
+                                           int32_t new_blk, int32_t tile, int32_t tuned) {
+    using namespace nsfrb;
+    if (!plan || dtype < NSFRB_F32 || dtype > NSFRB_F16 || n_items < 1 || new_blk < 0) return -1;
+    const nsfrb_config &c = plan->cfg;
+    SearchParams sp;
+    base_params(plan, sp);
+    // addresses that nothing reads: the choice looks at their alignment and at whether they are there
+    static char somewhere[64];
+    const uintptr_t base = (reinterpret_cast<uintptr_t>(somewhere) + 15) / 16 * 16;
+    sp.cube = reinterpret_cast<const void *>(base + offset);
+    sp.dtype = dtype;
+    sp.n_items = n_items;
+    sp.row_len = c.n_t;
+    sp.new_blk = new_blk;
+    if (new_blk > 0) {   // a ring row, its window start on the device
+        sp.row_len = static_cast<int64_t>(align_up(static_cast<size_t>(2 * c.n_t + 8), dtype == NSFRB_F32 ? 4 : 8));
+        sp.t_off_dev = reinterpret_cast<const int32_t *>(base);
+    }
+    if (c.out_mode == NSFRB_OUT_FULL) sp.full_snr = reinterpret_cast<float *>(base);
+    if (mad_slabs_apply(plan)) sp.noise_mode = NSFRB_NOISE_KNOWN;
+    size_t smem = 0;
+    if (!choose_stage_for(plan->C, 227 * 1024, sp, smem, tile, tuned != 0)) return 0;
+    if (sp.short_w > 0) return 4;
+    if (sp.mid_w > 0) return 5;
+    if (sp.wide) return 6;
+    if (sp.team) return 7;
+    if (sp.serve) return 8;
+    if (plan->C == kLongC) return 3;
+    return sp.pipe ? 2 : 1;
+}
+
 extern "C" nsfrb_status nsfrb_dbg_mad_normalise(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t,
                                                 float *d_out, uint8_t *d_bad, void *stream) {
     using namespace nsfrb;

@@ -133,7 +133,7 @@ bool tile_is_known(int t) {
     return false;
 }
 
-bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int tile_pref) {
+bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int tile_pref, bool tile_tuned) {
     // long windows whose pixels fit in shared memory: several warps to a DM row (figures beside the kernel)
     if (C == kLongC && choose_wide(sp, max_smem, smem)) return true;
     if (C == kLongC) {
@@ -147,8 +147,10 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
         smem = long_smem(sp, w);
         return true;
     }
-    // serving blocks of at most 32 samples: boxcars updated from row to row (figures beside the kernel)
-    if (tile_pref == 0 && choose_serve(sp, max_smem, smem)) return true;
+    // serving blocks of at most 32 samples: boxcars updated from row to row (figures beside the kernel), unless the
+    // caller chose a tile; one that autotune kept was timed on whole windows and says nothing of blocks
+    // (301 x 301 pixels of 1200 BF16 samples, 25-sample block: 1.88 ms, 3.30 ms with tile 41)
+    if ((tile_pref == 0 || tile_tuned) && choose_serve(sp, max_smem, smem)) return true;
     // windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel
     // is asked for: a lane per pixel instead of a warp per DM row.  301 x 301 pixels, FP32, against
     // the barrier-free kernel's best tile: 16 samples 71 us (1450), 32 samples 138 us (1488), 64
@@ -235,7 +237,7 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
 }
 
 bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem) {
-    return choose_stage_for(pl->C, pl->max_smem, sp, smem, pl->tile[sp.dtype]);
+    return choose_stage_for(pl->C, pl->max_smem, sp, smem, pl->tile[sp.dtype], pl->tile_tuned[sp.dtype]);
 }
 
 // records which tile the search launch of `sp` takes
@@ -770,6 +772,7 @@ nsfrb_status nsfrb_plan_set_tile(nsfrb_plan_t plan, int32_t dtype, int32_t tile)
     if (dtype < NSFRB_F32 || dtype > NSFRB_F16) return fail(plan, NSFRB_EINVAL, "unknown storage type");
     if (tile != 0 && !tile_is_known(tile)) return fail(plan, NSFRB_EINVAL, "unknown tile");
     plan->tile[dtype] = tile;
+    plan->tile_tuned[dtype] = false;
     return NSFRB_OK;
 }
 
@@ -840,6 +843,7 @@ nsfrb_status nsfrb_plan_autotune(nsfrb_plan_t plan, const void *d_cube, const fl
         }
     }
     plan->tile[s_t] = timed ? best : keep[s_t];
+    plan->tile_tuned[s_t] = plan->tile_tuned[s_t] || timed;
     if (h_tile) *h_tile = plan->tile[s_t];
     // the plan's results are those of a search with the chosen tile
     st = nsfrb_search(plan, d_cube, d_sigma, nullptr, stream);
