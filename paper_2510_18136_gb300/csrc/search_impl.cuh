@@ -1609,15 +1609,21 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(C, true)) search_kernel_
     // the team's items: it0 = CTA * TEAMS + team, then every G = grid * TEAMS
     const int64_t G = static_cast<int64_t>(gridDim.x) * TEAMS;
     const int64_t it0 = static_cast<int64_t>(blockIdx.x) * TEAMS + team;
+    int issued_last = -1;   // local index of the last item whose copy this warp started
     if (wt == 0) {
-        if (it0 < n_items) issue_warp(it0, slot0, 2 * team);
-        if (NB == 2 && it0 + G < n_items) issue_warp(it0 + G, slot0 + 1, 2 * team + 1);
+        if (it0 < n_items) {
+            issue_warp(it0, slot0, 2 * team);
+            issued_last = 0;
+        }
+        if (NB == 2 && it0 + G < n_items) {
+            issue_warp(it0 + G, slot0 + 1, 2 * team + 1);
+            issued_last = 1;
+        }
     }
 
     const int n_ua = p.n_u_active;
     float *Pw = s_pbuf + (size_t)warp * 32 * C;
     float *Sw = reinterpret_cast<float *>(smem + lay.fscr) + (size_t)warp * kFindScr;
-    int issued_last = -1;   // local index of the last item whose copy this warp started
     int i = 0;
     for (int64_t it = it0; it < n_items; it += G, ++i) {
         const int b = i % NB, sl = slot0 + b, rs = 2 * team + (i & 1);
@@ -1706,9 +1712,12 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(C, true)) search_kernel_
         }
         __syncwarp();
     }
-    // after an error: wait (bounded) for copies this warp started that may still be in flight
-    if (*reinterpret_cast<volatile int32_t *>(s_flag) && lane == 0 && issued_last >= 0)
+    // after an error: wait (bounded) for copies this warp started that may still be in flight (with two buffers
+    // also the one before the last, whose phase has passed where another warp started the next into it)
+    if (*reinterpret_cast<volatile int32_t *>(s_flag) && lane == 0 && issued_last >= 0) {
         mbar_wait(&s_bar[slot0 + issued_last % NB], static_cast<uint32_t>(issued_last / NB) & 1u);
+        if (NB == 2 && issued_last == 1) mbar_wait(&s_bar[slot0], 0u);
+    }
 }
 
 }  // namespace dev

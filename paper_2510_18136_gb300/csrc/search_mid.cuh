@@ -161,7 +161,10 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
         const int landed = p.stage == 1 ? mbar_wait(s_bar, phase) : 1;
         phase ^= 1u;
         if (!__syncthreads_and(landed)) {
-            if (tid == 0) atomicOr(p.err, ERR_WAIT_TIMEOUT);
+            if (tid == 0) {
+                atomicOr(p.err, ERR_WAIT_TIMEOUT);
+                mbar_wait(s_bar, phase ^ 1u);   // the copies in flight, bounded, before the CTA leaves
+            }
             return;
         }
 

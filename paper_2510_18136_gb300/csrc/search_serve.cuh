@@ -148,11 +148,14 @@ __global__ void __launch_bounds__(TEAMS * W * 32, 1) search_kernel_serve(const _
     __syncthreads();
     const int64_t G = static_cast<int64_t>(gridDim.x) * TEAMS;
     const int64_t it0 = static_cast<int64_t>(blockIdx.x) * TEAMS + team;
-    if (wt == 0 && it0 < n_items) issue_warp(it0, 2 * team);
+    int issued_last = -1;   // local index of the last item whose copy this warp started
+    if (wt == 0 && it0 < n_items) {
+        issue_warp(it0, 2 * team);
+        issued_last = 0;
+    }
 
     float *Pw = reinterpret_cast<float *>(smem + lay.pbuf) + (size_t)warp * 32 * C;
     const int t0 = lane * C;
-    int issued_last = -1;   // local index of the last item whose copy this warp started
     int i = 0;
     for (int64_t it = it0; it < n_items; it += G, ++i) {
         const int rs = 2 * team + (i & 1);
