@@ -45,6 +45,12 @@ nsfrb_status nsfrb_dbg_conv3(int32_t path, int32_t B, int32_t D, int32_t H, int3
  * if it did not, EINVAL for a bad limit.  Synchronous. */
 nsfrb_status nsfrb_dbg_wait_timeout(int32_t limit_ms);
 
+/* nsfrb_bin_time with the odd warps of every CTA taking the wait for its tile number give_up (counted from 0
+ * per CTA) as run out: that tile and the later ones are then read in place and nothing more is copied; the
+ * sums are those of nsfrb_bin_time, bit for bit.  give_up < 0: nsfrb_bin_time itself. */
+nsfrb_status nsfrb_dbg_bin_time(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, int32_t factor,
+                                int32_t give_up, float *d_out, void *stream);
+
 /* The MAD normalisation pass of the search (Sec. 2.2, robust reading) on its own, asynchronous on
  * `stream`: for each of the n_rows rows of n_t samples of d_in (`dtype` storage, row-major),
  *   m = median, MAD = median |x - m| (exact order statistics; for even n_t the mean of the two

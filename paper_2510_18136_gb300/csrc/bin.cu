@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include "async_copy.cuh"
+#include "nsfrb_debug.h"
 #include "plan_internal.h"
 
 namespace nsfrb {
@@ -55,12 +56,16 @@ constexpr int kBinTileFactor = 32;     // smallest factor
 // into `parts` runs, one thread each, thread part * outputs + output: a warp's lanes then read runs
 // `factor` samples apart, and where that stride shares a power of two with the banks, lane o starts its run
 // `rot` samples late (and wraps), so that the lanes spread over all banks.
+// Once a copy has not landed within its wait's limit, no other is started: this and every later tile is
+// read in place, and the copies in flight are waited for (bounded) before the CTA leaves.  give_up >= 0 (tests): the
+// odd warps take the wait for this CTA's tile give_up as run out.
 template <typename T>
 __global__ void __launch_bounds__(kBinThreads, 2)
 bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, int rows, int parts,
-                float *__restrict__ out) {
+                float *__restrict__ out, int give_up) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_full[kBinStages];
+    __shared__ int s_stuck;   // a wait has run out
     __shared__ float s_part[kBinThreads];
     const int n_out = n_t / factor;
     const uint32_t tile_bytes = static_cast<uint32_t>(rows) * n_t * sizeof(T);
@@ -71,6 +76,7 @@ bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, i
         dev::bulk_g2s(smem + static_cast<size_t>(st) * tile_bytes, in + tile * rows * n_t, tile_bytes, &s_full[st]);
     };
     if (tid == 0) {
+        s_stuck = 0;
         for (int st = 0; st < kBinStages; ++st) dev::mbar_init(&s_full[st], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         dev::fence_proxy_async();
@@ -122,17 +128,30 @@ bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, i
             }
         }
     };
-    int st = 0;
+    int st = 0, mine = 0;   // the tile's stage and ordinal among this CTA's
     uint32_t parity = 0;
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    bool stuck = false;
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++mine) {
         const T *src = reinterpret_cast<const T *>(smem + static_cast<size_t>(st) * tile_bytes);
-        // a copy that has not landed within the wait's limit: the tile is read in place
-        if (!dev::mbar_wait(&s_full[st], parity)) src = in + tile * rows * n_t;
+        if (stuck) {
+            src = in + tile * rows * n_t;
+        } else if ((mine == give_up && (tid & 32)) || !dev::mbar_wait(&s_full[st], parity)) {
+            src = in + tile * rows * n_t;
+            s_stuck = 1;
+        }
         sum_rows(src, tile * rows, rows);
         dev::fence_proxy_async();
         __syncthreads();   // the stage has been read
         const int64_t next = tile + static_cast<int64_t>(kBinStages) * gridDim.x;
-        if (tid == 0 && next < n_tiles) issue(next, st);
+        if (!stuck && s_stuck) {
+            stuck = true;
+            // copies of the tiles up to kBinStages - 1 ahead, this one's among them
+            if (tid == 0)
+                for (int o = mine; o < mine + kBinStages; ++o)
+                    if (blockIdx.x + static_cast<int64_t>(o) * gridDim.x < n_tiles)
+                        dev::mbar_wait(&s_full[o % kBinStages], static_cast<uint32_t>(o / kBinStages) & 1u);
+        }
+        if (tid == 0 && !stuck && next < n_tiles) issue(next, st);
         if (++st == kBinStages) {
             st = 0;
             parity ^= 1u;
@@ -143,7 +162,8 @@ bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, i
 }
 
 template <typename T>
-cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, float *d_out, cudaStream_t s) {
+cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, float *d_out, cudaStream_t s,
+                       int give_up) {
     const T *in = static_cast<const T *>(d_in);
     const int64_t total = n_rows * (n_t / factor);
     // rows per tile: whole 16-byte units of contiguous memory, up to a stage
@@ -165,13 +185,26 @@ cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, fl
         int parts = 1;   // threads per output, while they and the samples last
         while (parts < 32 && 2 * parts * rows * (n_t / factor) <= kBinThreads && factor >= 16 * parts) parts *= 2;
         const int grid = static_cast<int>(std::min<int64_t>(n_rows / rows, 2 * n_sm));
-        bin_tile_kernel<T><<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out);
+        bin_tile_kernel<T><<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out, give_up);
         return cudaGetLastError();
     }
     const int bs = 256;
     const int grid = static_cast<int>(std::min<int64_t>((total + bs - 1) / bs, 152 * 64));
     bin_kernel<T><<<grid, bs, 0, s>>>(in, n_rows, n_t, factor, d_out);
     return cudaGetLastError();
+}
+
+nsfrb_status bin_time(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, int32_t factor, float *d_out,
+                      void *stream, int give_up) {
+    if (!d_in || !d_out || n_rows < 0 || n_t < 1 || factor < 1 || factor > n_t || dtype < NSFRB_F32 ||
+        dtype > NSFRB_F16)
+        return fail(nullptr, NSFRB_EINVAL, "bad argument");
+    if (n_rows * (n_t / factor) == 0) return NSFRB_OK;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const cudaError_t e = dtype == NSFRB_F32    ? launch_bin<float>(d_in, n_rows, n_t, factor, d_out, s, give_up)
+                          : dtype == NSFRB_BF16 ? launch_bin<__nv_bfloat16>(d_in, n_rows, n_t, factor, d_out, s, give_up)
+                                                : launch_bin<__half>(d_in, n_rows, n_t, factor, d_out, s, give_up);
+    return cuda_check(nullptr, e, "bin launch");
 }
 
 }  // namespace
@@ -181,13 +214,10 @@ using namespace nsfrb;
 
 extern "C" nsfrb_status nsfrb_bin_time(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, int32_t factor,
                                        float *d_out, void *stream) {
-    if (!d_in || !d_out || n_rows < 0 || n_t < 1 || factor < 1 || factor > n_t || dtype < NSFRB_F32 ||
-        dtype > NSFRB_F16)
-        return fail(nullptr, NSFRB_EINVAL, "bad argument");
-    if (n_rows * (n_t / factor) == 0) return NSFRB_OK;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const cudaError_t e = dtype == NSFRB_F32    ? launch_bin<float>(d_in, n_rows, n_t, factor, d_out, s)
-                          : dtype == NSFRB_BF16 ? launch_bin<__nv_bfloat16>(d_in, n_rows, n_t, factor, d_out, s)
-                                                : launch_bin<__half>(d_in, n_rows, n_t, factor, d_out, s);
-    return cuda_check(nullptr, e, "bin launch");
+    return bin_time(d_in, dtype, n_rows, n_t, factor, d_out, stream, -1);
+}
+
+extern "C" nsfrb_status nsfrb_dbg_bin_time(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, int32_t factor,
+                                           int32_t give_up, float *d_out, void *stream) {
+    return bin_time(d_in, dtype, n_rows, n_t, factor, d_out, stream, give_up);
 }

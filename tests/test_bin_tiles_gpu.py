@@ -38,3 +38,27 @@ def test_bin_tiles(multiscale, dtype, n_pix, n_sub, n_t, factor):
     off.copy_(dev)
     got = multiscale.bin_time(off, factor).cpu().double()
     assert ((got - ref).abs() <= tol).all()
+
+
+@pytest.fixture(scope="module")
+def native(multiscale):
+    from paper_2510_18136_gb300 import native as nat
+    return nat
+
+
+@pytest.mark.parametrize("give_up", [0, 1, 4, 7, 12])
+@pytest.mark.parametrize("n_t,factor,dtype", [(1200, 75, torch.float32), (640, 32, torch.bfloat16), (1000, 1000, torch.float32)])
+def test_a_wait_that_runs_out_leaves_the_sums(native, n_t, factor, dtype, give_up):
+    """From a tile whose copy is given up the rows are read in place; enough rows for 13 tiles of each CTA."""
+    row = n_t * (4 if dtype == torch.float32 else 2)
+    n_rows = 13 * 304 * (20480 // row) + 5
+    x = torch.randn((n_rows, n_t), generator=torch.Generator("cuda").manual_seed(1), device="cuda").to(dtype)
+    want = torch.empty((n_rows, n_t // factor), device="cuda")
+    got = torch.full_like(want, float("nan"))
+    code = native.F32 if dtype == torch.float32 else native.BF16
+    for k, out in ((-1, want), (give_up, got)):
+        st = native.lib.nsfrb_dbg_bin_time(native._ptr(x), code, n_rows, n_t, factor, k, native._ptr(out),
+                                           native._stream_handle(None))
+        assert st == native.OK
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
