@@ -45,6 +45,11 @@ nsfrb_status nsfrb_dbg_conv3(int32_t path, int32_t B, int32_t D, int32_t H, int3
  * if it did not, EINVAL for a bad limit.  Synchronous. */
 nsfrb_status nsfrb_dbg_wait_timeout(int32_t limit_ms);
 
+/* Searches of the plan run the kernel made for the window's length wherever it fits, also where the default (tile 0)
+ * would take a general kernel because it is faster there (few pixels, few DM rows): for tests at
+ * sizes an oracle can follow.  EINVAL for a null plan. */
+nsfrb_status nsfrb_dbg_plan_by_length(nsfrb_plan_t plan, int32_t on);
+
 /* nsfrb_bin_time with the odd warps of every CTA taking the wait for its tile number give_up (counted from 0
  * per CTA) as run out: that tile and the later ones are then read in place and nothing more is copied; the
  * sums are those of nsfrb_bin_time, bit for bit.  give_up < 0: nsfrb_bin_time itself. */
@@ -60,10 +65,10 @@ nsfrb_status nsfrb_dbg_bin_time(const void *d_in, int32_t dtype, int64_t n_rows,
 nsfrb_status nsfrb_dbg_mad_normalise(const void *d_in, int32_t dtype, int64_t n_rows, int32_t n_t, float *d_out,
                                      uint8_t *d_bad, void *stream);
 
-/* The kernel that a search of n_items of the plan's pixels would run on a device with 227 KB of
+/* The kernel that a search would run, were the plan's image n_items pixels large, on a device with 227 KB of
  * shared memory per block, for rows stored as dtype at an address `offset` bytes past a multiple of
  * 16; new_blk > 0: a block of that many samples of a served window.  tile, tuned: the tile
- * that the plan would hold, and whether autotune kept it.  Host code only.  Returns 1 the
+ * that the plan would hold (-1: 0 after nsfrb_dbg_plan_by_length), and whether autotune kept it.  Host code only.  Returns 1 the
  * barrier kernel, 2 the barrier-free kernel, 3 the long-window kernel, 4 short, 5 mid, 6 wide,
  * 7 team, 8 serving; 0 where nothing fits, -1 for bad arguments. */
 int32_t nsfrb_dbg_search_kernel(nsfrb_plan_t plan, int32_t dtype, int64_t n_items, int32_t offset, int32_t new_blk,

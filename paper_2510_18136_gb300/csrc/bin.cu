@@ -177,16 +177,32 @@ cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, fl
         int dev_id = 0, n_sm = 0;
         cudaError_t e = cudaGetDevice(&dev_id);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev_id);
-        const int smem = kBinStages * rows * row_bytes;
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(bin_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kBinStages * kBinStageBytes);   // every call's limit: see raise_smem_limit
         if (e != cudaSuccess) return e;
+        const int n_out = n_t / factor, resident = 2 * n_sm;
+        const int64_t n_tiles = n_rows / rows;
         int parts = 1;   // threads per output, while they and the samples last
-        while (parts < 32 && 2 * parts * rows * (n_t / factor) <= kBinThreads && factor >= 16 * parts) parts *= 2;
-        const int grid = static_cast<int>(std::min<int64_t>(n_rows / rows, 2 * n_sm));
-        bin_tile_kernel<T><<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out, give_up);
-        return cudaGetLastError();
+        while (parts < 32 && 2 * parts * rows * n_out <= kBinThreads && factor >= 16 * parts) parts *= 2;
+        // In place all the same:
+        //  * fewer tiles than resident CTAs and a thread per output: a tile's chain of copy and sums takes longer
+        //    than the loads of as many threads over the whole chip (1024 rows of 100 samples by 33, FP32: 6.2 us by
+        //    tiles, 4.2 in place; 16384 rows of 64 BF16 samples by 32: 8.3 and 6.2), unless the factor is a
+        //    multiple of 64, where a load's lanes fall on the same banks of L1 (16 x 1200 BF16 by 64: 6.2, 10.3);
+        //  * many tiles of few outputs that leave a good part of the samples out: they are copied all the
+        //    same, and a quarter of the threads sum (65536 rows of 3000 FP32 samples by 1024: 435 us by
+        //    tiles, 271 in place; 4096 rows 33 and 78).
+        const bool few = parts == 1 && n_tiles < resident && factor % 64 != 0;
+        const bool loose = sizeof(T) == 4 && 4 * parts * rows * n_out <= kBinThreads &&
+                           4 * (n_t - n_out * factor) > n_t && n_tiles >= 40 * resident;
+        if (!few && !loose) {
+            // every call's limit: see raise_smem_limit
+            e = cudaFuncSetAttribute(bin_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kBinStages * kBinStageBytes);
+            if (e != cudaSuccess) return e;
+            const int smem = kBinStages * rows * row_bytes;
+            const int grid = static_cast<int>(std::min<int64_t>(n_tiles, resident));
+            bin_tile_kernel<T><<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out, give_up);
+            return cudaGetLastError();
+        }
     }
     const int bs = 256;
     const int grid = static_cast<int>(std::min<int64_t>((total + bs - 1) / bs, 152 * 64));

@@ -42,6 +42,12 @@ extern "C" nsfrb_status nsfrb_dbg_wait_timeout(int32_t limit_ms) {
     return (h_err & ERR_WAIT_TIMEOUT) ? NSFRB_ETIMEOUT : NSFRB_OK;
 }
 
+extern "C" nsfrb_status nsfrb_dbg_plan_by_length(nsfrb_plan_t plan, int32_t on) {
+    if (!plan) return NSFRB_EINVAL;
+    plan->by_length = on != 0;
+    return NSFRB_OK;
+}
+
 extern "C" int32_t nsfrb_dbg_search_kernel(nsfrb_plan_t plan, int32_t dtype, int64_t n_items, int32_t offset,
                                            int32_t new_blk, int32_t tile, int32_t tuned) {
     using namespace nsfrb;
@@ -54,7 +60,7 @@ extern "C" int32_t nsfrb_dbg_search_kernel(nsfrb_plan_t plan, int32_t dtype, int
     const uintptr_t base = (reinterpret_cast<uintptr_t>(somewhere) + 15) / 16 * 16;
     sp.cube = reinterpret_cast<const void *>(base + offset);
     sp.dtype = dtype;
-    sp.n_items = n_items;
+    sp.n_items = sp.n_pix = n_items;
     sp.row_len = c.n_t;
     sp.new_blk = new_blk;
     if (new_blk > 0) {   // a ring row, its window start on the device

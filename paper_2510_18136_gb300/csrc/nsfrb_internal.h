@@ -16,6 +16,7 @@ constexpr int kMaxSub = 32;               // subbands per plan
 constexpr int kMaxT = 4096;               // longest window
 constexpr int kMaxTRegs = 1247;           // longest window of the register path (32 lanes x 39 samples - 1)
 constexpr int kLongC = 128;               // "chunk" of longer windows: the long-window kernel
+constexpr int kSms = 152;                 // multiprocessors (lines of dispatch rules that depend on them)
 constexpr int kShortT = 64;               // longest window of the short-window kernel
 constexpr int kSmallMax = 16;             // widths <= min(C, 16) use the in-lane path
 constexpr int kHistBins = 256;            // radix-select digit bins (MAD mode)
@@ -97,6 +98,7 @@ struct SearchParams {
                            // pixel with its own buffers; long-window kernel: warps per CTA
     int32_t nb;            // barrier-free kernel: pixel buffers per team, 2 (the pixel after next
                            // copied while one is searched) or 1 (the next copied after a pixel)
+    int64_t n_pix;         // pixels of the plan (n_items: of this launch)
     int32_t short_w;       // > 0: the short-window kernel with this many warps per CTA
     int32_t mid_w, mid_c, mid_s;   // mid_w > 0: the mid-window kernel, warps per CTA, samples per lane,
                                    // lanes per pixel

@@ -115,6 +115,7 @@ void base_params(const nsfrb_plan_s *pl, SearchParams &sp) {
         }
     }
     sp.n_dm = c.n_dm;
+    sp.n_pix = static_cast<int64_t>(c.ny) * c.nx;
     sp.rec = pl->d_rec;
     sp.err = pl->d_err;
     if (c.out_mode == NSFRB_OUT_FULL) {
@@ -131,6 +132,53 @@ bool tile_is_known(int t) {
     for (const int k : kTileCodes)
         if (k == t) return true;
     return false;
+}
+
+// Windows up to 1215 samples that stay with the general kernels (search_impl.cuh), where those are the faster ones: by
+// the plan's pixels (whatever part of them a launch takes, so that slabs, re-scoring and a search of the whole
+// cube run the same kernel), its distinct DM rows and its subbands.  Of 9400 combinations measured (8 to
+// 1215 samples, 1 to 90601 pixels, 1 to 101 rows, 4 to 32 subbands, FP32 and BF16, cold L2):
+//  * Few pixels.  The kernels by window length put 2 to 32 pixels on a CTA and last about as long for one set of
+//    them as for one per SM; a CTA per pixel fills the chip sooner.  16 subbands, 64 pixels: 25 BF16 samples, 40
+//    rows 45 us against 16; 240 BF16, 40 rows 31 against 17.  The lines lie at the resident CTAs of the
+//    kernel replaced (three, two or one per SM by chunk size), where the barrier kernel would run; for 16-bit
+//    rows of up to 64 samples, whose widening copy is slow, at several times that.
+//  * Few rows of FP32 windows the barrier-free kernel takes: the work is the copy, which that kernel overlaps with
+//    the search.  301 x 301 pixels, one row: 64 samples 1.64 times its time, 240 1.66, 256 two rows
+//    1.42, eight rows 1.1, twelve 0.84; 500 twelve rows 1.06, sixteen 1.0; 32 samples one row 0.55.
+bool general_is_faster(const SearchParams &sp, int C) {
+    const int T = sp.n_t, K = sp.n_sub, u = sp.n_u_active, es = static_cast<int>(elem_size(sp.dtype));
+    const int64_t n = sp.n_pix, per = kSms;
+    const bool rows16 = T % (16 / es) == 0 && reinterpret_cast<uintptr_t>(sp.cube) % 16 == 0;
+    if (T > 1215 || u < 1) return false;
+    if (rows16 && sp.dtype != NSFRB_F32 && C % 2 == 0) return false;
+    if (rows16 && sp.dtype == NSFRB_F32) {   // the barrier-free kernel applies
+        if (T > 607) return false;
+        if (T > 207)
+            return (u < 12 && 4 * u < 3 * K) || (T > 415 && T <= 543 && u < K && u < 16 && n > 4 * per);
+        if (T > kShortT + 112) return 5 * u <= K;
+        if (T > kShortT)
+            return 10 * u <= K || (8 * u <= K && T > 80 && n <= 128 * per) || (5 * u <= K && n <= 3 * per);
+        if (T > 32)
+            return 10 * u <= K || (8 * u <= K && T > 48) || (2 * u <= K && n <= 9 * per) || (2 * u <= 3 * K && n <= 3 * per);
+        return (n <= 3 * per && 4 * u <= 3 * K && (T > 16 || 8 * u <= 3 * K)) || (n <= 7 * per && 5 * u <= K && T > 16);
+    }
+    if (T <= kShortT) {
+        if (es == 4) return n <= 3 * per;
+        return n <= (T > 8 && T <= 16 ? 5 : rows16 || T <= 20 || u >= 64 ? 8 : 11) * per;
+    }
+    int waves;
+    if (C <= 5)
+        waves = 3;
+    else if (C == 9)
+        waves = T > 207 ? 3 : 2;
+    else if (C == 17)
+        waves = rows16 ? (T > 415 ? 2 : 1) : (u >= 64 && (es == 2 || T > 415) ? 2 : 0);
+    else if (C == 25)
+        waves = rows16 ? (u >= 64 ? 2 : 1) : (u >= 64 && es == 2 ? 1 : 0);
+    else
+        waves = u >= 64 && es == 2 ? 1 : 0;
+    return n * std::max(K, 16) <= waves * 16 * per;   // more subbands: fewer sets of pixels fit
 }
 
 bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int tile_pref, bool tile_tuned) {
@@ -150,13 +198,13 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
     // serving blocks of at most 32 samples: boxcars updated from row to row (figures beside the kernel), unless the
     // caller chose a tile; one that autotune kept was timed on whole windows and says nothing of blocks
     // (301 x 301 pixels of 1200 BF16 samples, 25-sample block: 1.88 ms, 3.30 ms with tile 41)
-    if ((tile_pref == 0 || tile_tuned) && choose_serve(sp, max_smem, smem)) return true;
-    // windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel
-    // is asked for: a lane per pixel instead of a warp per DM row.  301 x 301 pixels, FP32, against
-    // the barrier-free kernel's best tile: 16 samples 71 us (1450), 32 samples 138 us (1488), 64
-    // samples 366 us (1570) at 16 DM, 39 (339), 79 (362) and 238 us (369) at one.  The line lies at 64
-    // samples because a thread holds a row and its prefix in registers (210 of 255 at 64).
-    if (const int w = tile_pref == 0 ? short_warps(sp, max_smem) : 0) {
+    if ((tile_pref <= 0 || tile_tuned) && choose_serve(sp, max_smem, smem)) return true;
+    // Windows of up to 64 samples with candidate records, unless a tile of the barrier-free kernel is asked for or a
+    // general kernel is faster: a lane per pixel instead of a warp per DM row.  301 x 301 pixels, FP32, 16 DM rows
+    // against the barrier-free kernel's best tile: 16 samples 0.10 of its time, 32 0.17, 64 0.43.  The line
+    // lies at 64 samples because a thread holds a row and its prefix in registers (198 of 255 at 64).
+    const bool by_length = tile_pref < 0 || (tile_pref == 0 && !general_is_faster(sp, C));
+    if (const int w = by_length ? short_warps(sp, max_smem) : 0) {
         sp.pipe = 0;
         sp.stage = 0;
         sp.short_w = w;
@@ -165,9 +213,9 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
     }
     // longer ones up to 607 samples: several pixels to a warp (figures and the line between the two
     // beside the kernel and choose_mid)
-    if (tile_pref == 0 && choose_mid(sp, max_smem, smem)) return true;
+    if (by_length && choose_mid(sp, max_smem, smem)) return true;
     // and up to 1215 samples: the barrier-free search with more warps (figures beside the kernel)
-    if (tile_pref == 0 && choose_team(sp, max_smem, smem)) return true;
+    if (by_length && choose_team(sp, max_smem, smem)) return true;
     const uintptr_t base = reinterpret_cast<uintptr_t>(sp.cube);
     const int n_t = sp.n_t;
     const int epv = 16 / static_cast<int>(elem_size(sp.dtype));   // samples per 16 bytes
@@ -237,7 +285,9 @@ bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int t
 }
 
 bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem) {
-    return choose_stage_for(pl->C, pl->max_smem, sp, smem, pl->tile[sp.dtype], pl->tile_tuned[sp.dtype]);
+    const int tile = pl->tile[sp.dtype];
+    return choose_stage_for(pl->C, pl->max_smem, sp, smem, tile == 0 && pl->by_length ? -1 : tile,
+                            pl->tile_tuned[sp.dtype]);
 }
 
 // records which tile the search launch of `sp` takes

@@ -26,6 +26,7 @@ struct nsfrb_plan_s {
     // barrier-free kernel pixel x DM tile (10 * teams + buffers per team) per storage type of the
     // searched rows (FP32, BF16, FP16); 0 = the first of the default order that fits
     int32_t tile[3] = {0, 0, 0};
+    bool by_length = false;   // tests: tile 0 is the kernel of the window's length where it fits, also where another is faster
     bool tile_tuned[3] = {false, false, false};   // kept by autotune for whole-window searches, not set by the caller
     int32_t last_tile = 0, last_tile_st = -1;   // tile and storage type of the last search launch
     bool last_other = false;                    // it ran another kernel than the barrier-free or barrier one
@@ -93,7 +94,7 @@ void destroy_stream_state(nsfrb_plan_s *pl);
 void base_params(const nsfrb_plan_s *pl, SearchParams &sp);
 bool mad_slabs_apply(const nsfrb_plan_s *pl);
 bool choose_stage(const nsfrb_plan_s *pl, SearchParams &sp, size_t &smem);
-// tile_tuned: tile_pref was kept by autotune for searches of whole windows, and gives way to the serving kernel
+// tile_pref -1: tile 0 without general_is_faster; tile_tuned: tile_pref was kept by autotune for searches of whole windows, and gives way to the serving kernel
 bool choose_stage_for(int C, int max_smem, SearchParams &sp, size_t &smem, int tile_pref = 0, bool tile_tuned = false);
 
 cudaError_t launch_search_c1(const SearchParams &, int, size_t, cudaStream_t);

@@ -11,13 +11,6 @@ bool choose_mid(SearchParams &p, int max_smem, size_t &smem) {
     if (p.n_t <= kShortT || p.full_snr || p.noise_mode != 0 || p.t_wrap || p.t_stride || p.t_off || p.t_off_dev ||
         p.new_blk || p.row_len != p.n_t || p.n_u_active < 1)
         return false;
-    // Few rows of long FP32 windows stay with the barrier-free kernel where its copies apply: the work is
-    // then the copy, which that kernel overlaps with the search (301 x 301 pixels, one DM: 400
-    // samples 467 us against 624 here, 500 479 against 709, 240 equal; 16 rows: 400 samples 1843
-    // against 1503, 500 1845 against 1895).
-    if (p.dtype == NSFRB_F32 && p.n_t > 271 && p.n_u_active < 12 && p.n_t % 4 == 0 &&
-        reinterpret_cast<uintptr_t>(p.cube) % 16 == 0)
-        return false;
     int C = 0, S = 0;
 #define NSFRB_MID_PICK(CC, SS)            \
     if (C == 0 && CC * SS > p.n_t) {      \
@@ -45,7 +38,12 @@ bool choose_mid(SearchParams &p, int max_smem, size_t &smem) {
             best_smem = sm;
         }
     }
-    if (best == 0) return false;
+    // FP32 pixels so large that few warps stay resident are left to the barrier-free kernel where its buffers hold more
+    // of them (24 subbands, 9000 pixels: 520 samples 52 rows 671 us against 471; from 544 samples on they
+    // do not: 32 subbands, 600 samples 544 us against 2118)
+    if (best == 0 || (best < 8 && p.dtype == NSFRB_F32 && p.n_t > 415 && p.n_t <= 543 && p.n_t % 4 == 0 &&
+                      reinterpret_cast<uintptr_t>(p.cube) % 16 == 0))
+        return false;
     p.pipe = 0;
     p.mid_c = C;
     p.mid_s = S;

@@ -121,6 +121,7 @@ def _load() -> ctypes.CDLL:
                             c_int32),
         "nsfrb_dbg_wait_timeout": ([c_int32], c_int32),
         "nsfrb_dbg_bin_time": ([P, c_int32, c_int64, c_int32, c_int32, c_int32, P, P], c_int32),
+        "nsfrb_dbg_plan_by_length": ([P, c_int32], c_int32),
         "nsfrb_dbg_search_kernel": ([P, c_int32, c_int64, c_int32, c_int32, c_int32, c_int32], c_int32),
         "nsfrb_dbg_mad_normalise": ([P, c_int32, c_int64, c_int32, P, P, P], c_int32),
         "nsfrb_destroy": ([P], None),

@@ -39,6 +39,7 @@ def _config(n_t, widths, n_dm=12):
 
 def _search(native, cfg, cube, sig, dtype):
     with native.Plan(cfg, dtype=dtype) as plan:
+        native.lib.nsfrb_dbg_plan_by_length(plan.handle, 1)   # few pixels: general kernels are faster
         plan.search(cube.cuda(), torch.as_tensor(sig).cuda())
         return plan.best()
 

@@ -51,6 +51,7 @@ def test_searches_of_two_plans(native, n_t, noise):
         def run():
             s = torch.cuda.Stream()
             with native.Plan(cfg, noise=noise) as plan:
+                native.lib.nsfrb_dbg_plan_by_length(plan.handle, 1)   # few pixels: general kernels are faster
                 for _ in range(400):
                     plan.search(cube, stream=s)
                 got.append(plan.best()[0])

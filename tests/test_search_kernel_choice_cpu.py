@@ -34,6 +34,29 @@ def test_kernels_by_window_length(native):
     assert kernel(native, 1200, offset=4) == BARRIER and kernel(native, 25, offset=4) == SHORT
 
 
+@pytest.mark.parametrize("n_t,dtype,n_items,n_dm,want", [
+    # few pixels: 16-bit rows and FP32 rows off 16 bytes stay with the barrier kernel
+    (25, "bf16", 64, 64, BARRIER), (25, "bf16", 1672, 16, BARRIER), (25, "bf16", 1673, 16, SHORT),
+    (25, "f32", 456, 16, BARRIER), (25, "f32", 457, 16, SHORT), (240, "bf16", 456, 64, BARRIER),
+    (240, "bf16", 457, 64, MID), (640, "bf16", 152, 64, BARRIER), (640, "bf16", 153, 64, TEAM),
+    # FP32 rows of whole 16 bytes: by pixels and rows
+    (64, "f32", 90601, 1, FREE), (64, "f32", 90601, 64, SHORT), (32, "f32", 90601, 1, SHORT),
+    (32, "f32", 456, 1, FREE), (240, "f32", 90601, 1, FREE), (240, "f32", 90601, 64, MID), (160, "f32", 64, 64, MID),
+    (500, "f32", 90601, 12, FREE), (1200, "f32", 1, 1, TEAM), (1200, "bf16", 1, 1, TEAM), (1248, "f32", 1, 1, WIDE),
+])
+def test_few_pixels_and_few_rows(native, n_t, dtype, n_items, n_dm, want):
+    """The general kernels keep the calls they are faster at; a test's switch passes the rule by."""
+    hi = 0.0 if n_dm == 1 else 2000.0 if n_dm != 12 else 1500.0
+    assert kernel(native, n_t, dtype, n_items=n_items, n_dm=n_dm, dm_hi=hi) == want
+    assert kernel(native, n_t, dtype, n_items=n_items, n_dm=n_dm, dm_hi=hi, tile=-1) in (SHORT, MID, TEAM, WIDE)
+
+
+def test_a_wide_field_of_many_subbands(native):
+    """FP32 pixels too large for eight resident warps of the mid kernel, where the barrier-free kernel holds more."""
+    assert kernel(native, 520, n_sub=24, n_items=9000) == FREE
+    assert kernel(native, 600, n_sub=32, n_items=9000) == MID
+
+
 def test_a_tile_kept_by_autotune_leaves_serving_blocks_their_kernel(native):
     for dtype in ("f32", "bf16"):
         assert kernel(native, 1200, dtype, new_blk=25) == SERVE
