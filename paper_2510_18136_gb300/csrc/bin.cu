@@ -7,8 +7,8 @@
 // shared-memory stages by bulk copies and sums from there; bin_kernel reads global memory in place
 // and takes small factors and what the copies cannot (a cube off a 16-byte boundary, rows too long for
 // a stage).  In place, the 32 lanes of a load of the 75-fold sums touch 32 lines, and L1 rather than
-// HBM sets the rate: 301 x 301 x 16 rows of 1200 FP32 samples take 2301 us in place and 1028 us
-// through the tiles (6.86 TB/s); BF16 1962 and 700 us.
+// HBM sets the rate: 301 x 301 x 16 rows of 1200 FP32 samples take 2301 us in place and 1066 us
+// through the tiles (6.6 TB/s); BF16 1962 and 700 us.
 #include <algorithm>
 #include <numeric>
 
@@ -56,16 +56,15 @@ constexpr int kBinTileFactor = 32;     // smallest factor
 // into `parts` runs, one thread each, thread part * outputs + output: a warp's lanes then read runs
 // `factor` samples apart, and where that stride shares a power of two with the banks, lane o starts its run
 // `rot` samples late (and wraps), so that the lanes spread over all banks.
-// Once a copy has not landed within its wait's limit, no other is started: this and every later tile is
-// read in place, and the copies in flight are waited for (bounded) before the CTA leaves.  give_up >= 0 (tests): the
-// odd warps take the wait for this CTA's tile give_up as run out.
-template <typename T>
+// Once a copy has not landed within its wait's limit, no other is started: this tile (whose sums are written again) and
+// every later one is read in place, and the copies in flight are waited for (bounded) before the CTA leaves.  TEST: the odd
+// warps take the wait for this CTA's tile give_up as run out (looked at in the loop of the others it costs 5 %).
+template <typename T, bool TEST>
 __global__ void __launch_bounds__(kBinThreads, 2)
 bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, int rows, int parts,
                 float *__restrict__ out, int give_up) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_full[kBinStages];
-    __shared__ int s_stuck;   // a wait has run out
     __shared__ float s_part[kBinThreads];
     const int n_out = n_t / factor;
     const uint32_t tile_bytes = static_cast<uint32_t>(rows) * n_t * sizeof(T);
@@ -76,7 +75,6 @@ bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, i
         dev::bulk_g2s(smem + static_cast<size_t>(st) * tile_bytes, in + tile * rows * n_t, tile_bytes, &s_full[st]);
     };
     if (tid == 0) {
-        s_stuck = 0;
         for (int st = 0; st < kBinStages; ++st) dev::mbar_init(&s_full[st], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         dev::fence_proxy_async();
@@ -130,35 +128,38 @@ bin_tile_kernel(const T *__restrict__ in, int64_t n_rows, int n_t, int factor, i
     };
     int st = 0, mine = 0;   // the tile's stage and ordinal among this CTA's
     uint32_t parity = 0;
-    bool stuck = false;
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++mine) {
-        const T *src = reinterpret_cast<const T *>(smem + static_cast<size_t>(st) * tile_bytes);
-        if (stuck) {
-            src = in + tile * rows * n_t;
-        } else if ((mine == give_up && (tid & 32)) || !dev::mbar_wait(&s_full[st], parity)) {
-            src = in + tile * rows * n_t;
-            s_stuck = 1;
-        }
-        sum_rows(src, tile * rows, rows);
+    int64_t tile = blockIdx.x;
+    for (; tile < n_tiles; tile += gridDim.x, ++mine) {
+        bool stuck = false;
+        if constexpr (TEST) stuck = mine == give_up && (tid & 32);
+        if (!stuck) stuck = !dev::mbar_wait(&s_full[st], parity);
+        sum_rows(reinterpret_cast<const T *>(smem + static_cast<size_t>(st) * tile_bytes), tile * rows, rows);
         dev::fence_proxy_async();
-        __syncthreads();   // the stage has been read
+        if (__syncthreads_or(stuck)) break;   // (the stage has been read)
         const int64_t next = tile + static_cast<int64_t>(kBinStages) * gridDim.x;
-        if (!stuck && s_stuck) {
-            stuck = true;
-            // copies of the tiles up to kBinStages - 1 ahead, this one's among them
-            if (tid == 0)
-                for (int o = mine; o < mine + kBinStages; ++o)
-                    if (blockIdx.x + static_cast<int64_t>(o) * gridDim.x < n_tiles)
-                        dev::mbar_wait(&s_full[o % kBinStages], static_cast<uint32_t>(o / kBinStages) & 1u);
-        }
-        if (tid == 0 && !stuck && next < n_tiles) issue(next, st);
+        if (tid == 0 && next < n_tiles) issue(next, st);
         if (++st == kBinStages) {
             st = 0;
             parity ^= 1u;
         }
     }
+    if (tile < n_tiles && tid == 0)
+        // copies of the tiles up to kBinStages - 1 ahead, this one's among them
+        for (int o = mine; o < mine + kBinStages; ++o)
+            if (blockIdx.x + static_cast<int64_t>(o) * gridDim.x < n_tiles)
+                dev::mbar_wait(&s_full[o % kBinStages], static_cast<uint32_t>(o / kBinStages) & 1u);
+    // in place: the tiles left after a wait that ran out, and the last CTA the rows that fill no tile
     const int64_t left = n_tiles * rows;
-    if (left < n_rows && blockIdx.x == gridDim.x - 1) sum_rows(in + left * n_t, left, static_cast<int>(n_rows - left));
+    bool rest = left < n_rows && blockIdx.x == gridDim.x - 1;
+    while (tile < n_tiles || rest) {
+        const bool whole = tile < n_tiles;
+        const int64_t row = whole ? tile * rows : left;
+        sum_rows(in + row * n_t, row, whole ? rows : static_cast<int>(n_rows - left));
+        if (whole)
+            tile += gridDim.x;
+        else
+            rest = false;
+    }
 }
 
 template <typename T>
@@ -194,13 +195,13 @@ cudaError_t launch_bin(const void *d_in, int64_t n_rows, int n_t, int factor, fl
         const bool loose = sizeof(T) == 4 && 4 * parts * rows * n_out <= kBinThreads &&
                            4 * (n_t - n_out * factor) > n_t && n_tiles >= 40 * resident;
         if (!few && !loose) {
+            const auto kernel = give_up < 0 ? bin_tile_kernel<T, false> : bin_tile_kernel<T, true>;
             // every call's limit: see raise_smem_limit
-            e = cudaFuncSetAttribute(bin_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kBinStages * kBinStageBytes);
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBinStages * kBinStageBytes);
             if (e != cudaSuccess) return e;
             const int smem = kBinStages * rows * row_bytes;
             const int grid = static_cast<int>(std::min<int64_t>(n_tiles, resident));
-            bin_tile_kernel<T><<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out, give_up);
+            kernel<<<grid, kBinThreads, smem, s>>>(in, n_rows, n_t, factor, rows, parts, d_out, give_up);
             return cudaGetLastError();
         }
     }
