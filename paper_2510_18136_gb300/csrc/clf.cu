@@ -1227,7 +1227,10 @@ nsfrb_status nsfrb_clf_cutouts(nsfrb_plan_t plan, const void *d_cube, const floa
     cp.ny = c.ny, cp.nx = c.nx, cp.n_sub = c.n_sub, cp.n_t = c.n_t;
     cp.n = n, cp.D = d, cp.H = h, cp.W = w;
     cp.xt = std::min(w, std::max(1, kCutCols / c.n_sub));
-    const int64_t tiles = static_cast<int64_t>(n) * h * ((w + cp.xt - 1) / cp.xt) * ((d + kCutZ - 1) / kCutZ);
+    auto tiles_of = [&](int xt) { return static_cast<int64_t>(n) * h * ((w + xt - 1) / xt) * ((d + kCutZ - 1) / kCutZ); };
+    // few cutouts: narrower tiles, until there are enough for the resident CTAs (four per SM)
+    while (cp.xt > 2 && tiles_of(cp.xt) < 4 * kSms) cp.xt = (cp.xt + 1) / 2;
+    const int64_t tiles = tiles_of(cp.xt);
     const int grid = static_cast<int>(std::min<int64_t>(tiles, 1 << 20));
     const size_t smem = sizeof(uint16_t) * kCutZ * cut_pitch(cp.xt * c.n_sub);
     cudaStream_t s = static_cast<cudaStream_t>(stream);

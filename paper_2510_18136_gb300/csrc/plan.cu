@@ -160,7 +160,8 @@ bool general_is_faster(const SearchParams &sp, int C) {
         if (T > kShortT)
             return 10 * u <= K || (8 * u <= K && T > 80 && n <= 128 * per) || (5 * u <= K && n <= 3 * per);
         if (T > 32)
-            return 10 * u <= K || (8 * u <= K && T > 48) || (2 * u <= K && n <= 9 * per) || (2 * u <= 3 * K && n <= 3 * per);
+            return 10 * u <= K || (8 * u <= K && T > 48) || (2 * u <= K && n <= 9 * per) || (2 * u <= 3 * K && n <= 3 * per) ||
+                   (u <= 3 * K && n <= 2 * per && T > 48);
         return (n <= 3 * per && 4 * u <= 3 * K && (T > 16 || 8 * u <= 3 * K)) || (n <= 7 * per && 5 * u <= K && T > 16);
     }
     if (T <= kShortT) {
