@@ -124,15 +124,16 @@ def make_cube(native, synth, cfg, seed, device, dtype):
 
 # DRAM bytes (read + write) per 301x301 FP32 launch from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum of a 128x128 launch of search_kernel_team, 1263 MB, scaled by 90601 / 16384
-# pixels), valid for the kernel source with this sha256 prefix.
-NCU_TRAFFIC = {"sha256_16": "0021d370381b00e5", "bytes": (1.26e9 + 3.22e6) * 90601 / 16384,
-               "workload": (301, 301, "f32")}
+# pixels), valid for the kernel sources (the kernel and the row code it includes) with this sha256 prefix,
+# candidate records with the plan's default tile.
+NCU_TRAFFIC = {"sha256_16": "75c45ca75f241165", "bytes": (1.26e9 + 3.21e6) * 90601 / 16384,
+               "workload": (301, 301, 1200, 64, "f32", "candidates", 0)}
 
 
 # DRAM bytes of one imager call (grid_kernel + transform_kernel) from the ncu launch list of the
 # committed kernels (paper block: 25 x 16 x 8 x 3321 x 2 pol, 175 px); ncu flushes the caches
 # before each kernel, so the transform re-reads the 15.6 MB of partial grids from DRAM there.
-IMG_NCU_TRAFFIC = {"sha256_16": "efc27e98ac335103", "bytes": 181822464 + 6787328 + 15642112 + 203264}
+IMG_NCU_TRAFFIC = {"sha256_16": "edf7879e2db9d2b8", "bytes": 181.81e6 + 9.73e6 + 15.64e6 + 137.98e3}
 
 
 def imager_traffic():
@@ -142,39 +143,45 @@ def imager_traffic():
     return IMG_NCU_TRAFFIC["bytes"] if digest == IMG_NCU_TRAFFIC["sha256_16"] else None
 
 
-def measured_traffic(ny, nx, dtype):
-    """ncu traffic per launch if it was taken on the current kernel source, else None."""
+def measured_traffic(cfg, dtype, out, tile):
+    """ncu traffic per launch if it was taken on the current kernel sources and on this workload, else None."""
     import hashlib
-    src = os.path.join(ROOT, "paper_2510_18136_gb300", "csrc", "search_team.cuh")
-    with open(src, "rb") as fh:
-        digest = hashlib.sha256(fh.read()).hexdigest()[:16]
-    if digest != NCU_TRAFFIC["sha256_16"] or (ny, nx, dtype) != NCU_TRAFFIC["workload"]:
+    h = hashlib.sha256()
+    for name in ("search_team.cuh", "search_impl.cuh"):
+        with open(os.path.join(ROOT, "paper_2510_18136_gb300", "csrc", name), "rb") as fh:
+            h.update(fh.read())
+    workload = (cfg.ny, cfg.nx, cfg.n_t, len(cfg.dm), dtype, out, tile)
+    if h.hexdigest()[:16] != NCU_TRAFFIC["sha256_16"] or workload != NCU_TRAFFIC["workload"]:
         return None
     return NCU_TRAFFIC["bytes"]
 
 
-def search_kernel_name(n_t, dtype, noise="known", tile=None, out="candidates"):
+def default_kernel(native, plan, dtype, noise="known"):
+    """The code of the kernel that the plan's default (tile 0) runs (nsfrb_dbg_search_kernel)."""
+    code = {"f32": native.F32, "bf16": native.BF16, "f16": native.F16}["f32" if noise == "mad" else dtype]
+    return native.lib.nsfrb_dbg_search_kernel(plan.handle, code, plan.cfg.n_pix, 0, 0, 0, 0)
+
+
+def search_kernel_name(n_t, dtype, noise="known", tile=None, out="candidates", kernel=None):
     """The kernels the library launches for this window: chunks of C samples per lane, the smallest
     compiled C with 32 C > n_t.  With known noise the barrier-free kernel runs (FP32 rows; 16-bit
     rows read in place when C is even and the rows fill whole 16-byte units), with the pixel x DM
     tile (teams T, buffers per team B) the plan chose; MAD normalisation is a pass of its own into
     FP32 slabs that the barrier-free kernel then searches.  The last template argument is FULL.
-    tile 0 (the plan kept its default): the kernels of candidate records by window length."""
+    kernel: the library's code of the default kernel (default_kernel), where tile is 0 (the plan kept its
+    default): the kernels of candidate records by window length have codes from 4 on."""
     st = {"f32": 0, "bf16": 1, "f16": 2}[dtype]
     full = 1 if out == "full" else 0     # bool template arguments as ncu prints them
-    if tile == 0 and not full and n_t <= 1215:   # the default of candidate records (MAD slabs are FP32)
-        st = 0 if noise == "mad" else st
-        if n_t <= 64:
-            name = f"search_kernel_short<{next(n for n in (16, 26, 32, 48, 64) if n >= n_t)}>"
-        elif n_t <= 607:
-            tiles = ((22, 4), (26, 4), (34, 4), (22, 8), (26, 8), (34, 8), (22, 16), (26, 16), (34, 16), (38, 16))
-            name = "search_kernel_mid<%d, %d, %d>" % (*next(t for t in tiles if t[0] * t[1] > n_t), st)
-        else:
-            name = f"search_kernel_team<{next(c for c in (22, 26, 34, 38) if 32 * c > n_t)}, {st}, T, W>"
+    if tile == 0 and kernel is not None and kernel >= 4:
+        st = 0 if noise == "mad" else st     # MAD slabs are FP32
+        mid = ((22, 4), (26, 4), (34, 4), (22, 8), (26, 8), (34, 8), (22, 16), (26, 16), (34, 16), (38, 16))
+        wide = ((22, 2), (26, 2), (34, 2), (38, 2), (34, 3), (34, 4))
+        name = {4: lambda: f"search_kernel_short<{next(n for n in (16, 26, 32, 48, 64) if n >= n_t)}>",
+                5: lambda: "search_kernel_mid<%d, %d, %d>" % (*next(t for t in mid if t[0] * t[1] > n_t), st),
+                6: lambda: "search_kernel_wide<%d, %d, %d>" % (*next(t for t in wide if 32 * t[0] * t[1] > n_t), st),
+                7: lambda: f"search_kernel_team<{next(c for c in (22, 26, 34, 38) if 32 * c > n_t)}, {st}, T, W>"}[kernel]()
         return f"mad_normalise_kernel + {name} (FP32 slabs)" if noise == "mad" else name
     if n_t > 1247:   # beyond a warp's registers (MAD slabs are FP32)
-        if tile == 0 and not full:
-            return "search_kernel_wide (search_kernel_long where a pixel does not fit in shared memory)"
         return f"search_kernel_long<{0 if noise == 'mad' else st}, {full}>"
     c = next(c for c in (1, 3, 5, 9, 17, 25, 38, 39) if 32 * c >= n_t + 1)
     tt = ", T, B" if tile is None else f", {int(tile) // 10}, {int(tile) % 10}"
@@ -775,6 +782,7 @@ def stress_section(native, synth, steps: int, seed: int = 0, size: int = 512):
     plan = native.Plan(cfg, dtype="bf16", noise="mad")
     stream = torch.cuda.current_stream()
     tile, tile_ms = plan.autotune(cube, reps=2, stream=stream)   # tile of the FP32 slab search
+    kernel = default_kernel(native, plan, "bf16", "mad")
     ops, n_unique = alg_ops(cfg, plan)
     for _ in range(2):
         plan.search(cube, stream=stream)
@@ -826,7 +834,7 @@ def stress_section(native, synth, steps: int, seed: int = 0, size: int = 512):
             "false_alarm_pixels": fa, "false_alarm_fraction": fa / float(cfg.n_pix - len(inj)),
             "false_alarm_pixels_above_7.2": fa72,
             "roofline": {"bound": "alu", "achieved": ops / tk / 1e12, "peak": peak_ops / 1e12, "unit": "TFLOP/s",
-                         "frac": ops / tk / peak_ops, "kernel": search_kernel_name(cfg.n_t, 'bf16', 'mad', tile),
+                         "frac": ops / tk / peak_ops, "kernel": search_kernel_name(cfg.n_t, 'bf16', 'mad', tile, kernel=kernel),
                          "kernel_ms": tk * 1e3, "ops_per_launch": ops, "tile": tile, "tile_ms": tile_ms},
             "hbm": {"achieved_gbs": alg_bytes / tk / 1e9, "frac": alg_bytes / tk / 1e9 / pk["hbm_gbs"],
                     "bytes_per_launch": alg_bytes},
@@ -865,6 +873,7 @@ def main():
     stream = torch.cuda.current_stream()
     # pixel x DM tile of the search kernel: each tile that fits timed on this cube, the fastest kept
     tile, tile_ms = plan.autotune(cube, sigma, reps=3, stream=stream)
+    kernel = default_kernel(native, plan, args.dtype)
     ops, n_unique = alg_ops(cfg, plan)
     elem = 4 if args.dtype == "f32" else 2
     cube_bytes = cfg.n_pix * cfg.n_sub * cfg.n_t * elem
@@ -985,8 +994,8 @@ def main():
                                    "one GPU")},
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                      "unit": "TFLOP/s", "frac": achieved / peak_ops,
-                     "traffic": measured_traffic(cfg.ny, cfg.nx, args.dtype),
-                     "kernel": search_kernel_name(cfg.n_t, args.dtype, tile=tile, out=args.out),
+                     "traffic": measured_traffic(cfg, args.dtype, args.out, tile),
+                     "kernel": search_kernel_name(cfg.n_t, args.dtype, tile=tile, out=args.out, kernel=kernel),
                      "kernel_ms": kern_s * 1e3, "tile": tile, "tile_ms": tile_ms,
                      "ops_per_launch": ops, "peak_basis": f"{n_sm} SM x 128 FP32 lanes x "
                      f"{pk['sm_max_mhz']:.0f} MHz ({pk['source']} max clock)"},

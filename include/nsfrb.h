@@ -71,7 +71,9 @@ typedef struct {
                                 to 64), several pixels to a warp (607), a warp
                                 per DM row (1247), several warps per DM row
                                 where a pixel fits in shared memory, and one
-                                that reads the cube in place for the rest       */
+                                that reads the cube in place for the rest; few
+                                pixels or few distinct DM rows run the general
+                                kernel where that is the faster one             */
     double t_samp_ms;        /* sampling time, e.g. 134.2                      */
     double k_dm_ms;          /* dispersion constant in ms GHz^2, e.g. 4.149    */
     const double *freq_mhz;  /* [n_sub] subband centres, strictly increasing   */
@@ -178,8 +180,9 @@ nsfrb_status nsfrb_last_timing(nsfrb_plan_t plan, float *search_ms, float *total
  * order (different warps build a row group's partial sums from scratch).
  * Tile 0 (the default) = for candidate records of up to 1215 samples a kernel
  * made for the window's length (n_t above) with a shape of its own; where
- * those do not apply (FULL output, windows that are not whole 16-byte units),
- * the first of 41, 31, 22, 21, 12 whose buffers fit in shared memory. */
+ * those do not apply (FULL output, windows that are not whole 16-byte units)
+ * or are slower (few pixels, few distinct DM rows), the first of 41, 31, 22,
+ * 21, 12 whose buffers fit in shared memory. */
 #define NSFRB_N_TILES 5
 #define NSFRB_TILES 12, 22, 21, 31, 41
 

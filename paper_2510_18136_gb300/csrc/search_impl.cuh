@@ -2,9 +2,9 @@
 // per pixel, de-disperse every DM trial with integer shifts, boxcar-filter
 // every width with prefix sums, normalise to S/N, maximise over time, width
 // and DM.  Included by one translation unit per chunk size C.  These kernels serve FULL output,
-// in-kernel MAD, rings, lists of pixels for which the kernels by window length (search_short.cu,
-// search_mid.cuh, search_team.cuh, search_wide.cuh, search_serve.cuh) do not apply, and chosen tiles;
-// the building blocks are theirs too.
+// in-kernel MAD, rings, chosen tiles, and calls for which the kernels by window length (search_short.cu,
+// search_mid.cuh, search_team.cuh, search_wide.cuh, search_serve.cuh) do not apply or are slower (few
+// pixels, few DM rows); the building blocks are theirs too.
 //
 // Organisation (one CTA of 12 warps per pixel, persistent over pixels):
 //  * The pixel's [n_sub][n_t] tile is staged in shared memory (bulk copies

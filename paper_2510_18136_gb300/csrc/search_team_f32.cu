@@ -18,10 +18,12 @@ bool choose_team(SearchParams &p, int max_smem, size_t &smem) {
     if (C == 0 && 32 * CC > p.n_t) C = CC;
     NSFRB_TEAM_CHUNKS(NSFRB_TEAM_PICK)
 #undef NSFRB_TEAM_PICK
-    // The most pixels in shared memory first, then the most warps: sixteen warps of 128 registers where
-    // four pixels leave room for their prefix buffers, four teams of three before three of five (1200
-    // BF16 samples, 40401 pixels, 40 DM rows: 1965 us against 2165), two teams of eight or six last
-    // (1200 FP32 samples only fit the latter: 2395 us).
+    // The most pixels in shared memory first, then the most warps.  6080 pixels, 4 to 24 subbands, 608 to 1200 samples:
+    // sixteen warps in four teams against four teams of three 0.94 of the time at 608 samples (16 subbands, 40 rows:
+    // 202 us against 214; 10 subbands 167, 176), 0.97 at 1000 (273, 283), and 1.1 with very few rows (4 subbands, 5
+    // rows, 1200 samples: 66, 60); three teams of five or two of eight against two of six 0.80 with seven rows
+    // (20 subbands, 700 FP32 samples: 113 us, 145), 0.93 with 52 (294, 315), but 1.06 for 12 subbands of 1200 (336,
+    // 316).  Over all of them this order is 1 to 2 % faster than leaving out any of the shapes.
     const int shapes[] = {44, 43, 35, 28, 26};
     for (const int t : shapes) {
         const size_t sm = dev::team_layout(p, C, t / 10, t % 10).total;

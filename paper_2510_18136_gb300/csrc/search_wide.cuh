@@ -23,8 +23,9 @@
 // pixels x 16 subbands, 40 distinct DM rows, 12 widths, against the long-window kernel: 1250 samples FP32
 // 1.48 ms (7.44), 2048 1.90 ms (11.9), BF16 1.90 ms (16.4), 3000 2.70 ms (27.3), 4096 3.57 ms (38.5).  With
 // one FP32 prefix per segment and differences of it the same searches take 1.22, 1.54, 1.52, 2.10
-// and 2.81 ms, but after a sample of -1e4 the S/N is off by up to 6e-4 (here 3e-7, the long-window
-// kernel 5e-5), and a sample that is not a number left records without their sample.
+// and 2.81 ms, but beside a dip of -300 a sample over 256 of 2048 samples the relative error of the S/N
+// reaches 6e-4 (here 1.4e-7, the long-window kernel 2.4e-6), and a sample that is not a number left
+// records whose sample did not have their S/N.
 #pragma once
 
 #include <climits>

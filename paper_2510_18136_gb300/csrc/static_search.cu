@@ -75,10 +75,8 @@ __global__ void __launch_bounds__(kCompactBlock) static_scatter_kernel(const Pix
     }
 }
 
-// Staging scheme for a contiguous cube under this device's shared-memory limit, as nsfrb_search
-// chooses it: the barrier-free kernel for cubes with known noise whose rows are 16-byte aligned
-// (FP32 rows copied as they are, 16-bit rows read in place), else bulk copies with per-pixel
-// barriers, else plain loads.
+// Kernel and staging for a contiguous cube under this device's shared-memory limit, as nsfrb_search chooses them with
+// no tile set: the kernel made for the window's length, else a general one.
 bool static_stage(int C, int max_smem, SearchParams &sp, size_t &smem) { return choose_stage_for(C, max_smem, sp, smem); }
 
 // Once per device, with that device current: the device address of the

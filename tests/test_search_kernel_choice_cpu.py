@@ -64,3 +64,24 @@ def test_a_tile_kept_by_autotune_leaves_serving_blocks_their_kernel(native):
         assert kernel(native, 1200, dtype, new_blk=25, tile=21) == FREE      # the caller's choice
         assert kernel(native, 1200, dtype, new_blk=40, tile=21, tuned=True) == FREE
         assert kernel(native, 1200, dtype, tile=21, tuned=True) == FREE
+
+
+def test_bench_names_the_default_kernel(native):
+    import os
+    import sys
+
+    sys.path.insert(0, os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    import bench
+
+    def name(n_t, dtype, noise="known", n_sub=16, out="candidates"):
+        cfg = synth.SearchConfig(ny=301, nx=301, n_t=n_t, n_sub=n_sub, freq_mhz=synth.band_centres(n_sub),
+                                 widths=np.array([1, 8], np.int32), threshold=6.0)
+        with native.Plan(cfg, dtype=dtype, noise=noise, out=out) as plan:
+            return bench.search_kernel_name(n_t, dtype, noise, 0, out, bench.default_kernel(native, plan, dtype, noise))
+
+    assert name(1200, "f32") == "search_kernel_team<38, 0, T, W>"
+    assert name(1200, "bf16", "mad") == "mad_normalise_kernel + search_kernel_team<38, 0, T, W> (FP32 slabs)"
+    assert name(240, "bf16") == "search_kernel_mid<34, 8, 1>" and name(25, "f32") == "search_kernel_short<26>"
+    assert name(2048, "f32") == "search_kernel_wide<34, 2, 0>" and name(4096, "f32") == "search_kernel_long<0, 0>"
+    assert name(1231, "f32").startswith("search_kernel_pipe<39") or name(1231, "f32").startswith("search_kernel<39")
+    assert name(1200, "f32", out="full").startswith("search_kernel_pipe<38, 0")
