@@ -19,14 +19,16 @@
 //    P[t + w] is a register of the same lane for every power of two w >= 2 S.
 //  * Each lane tracks its own best (S/N, row, width) over all rows: no warp maxima per row.  At the end
 //    a warp per pixel rebuilds the best row from all subbands, and takes the record's S/N and the
-//    earliest sample reaching it from that row, with the same two forms of boxcars.
+//    earliest sample reaching it from that row: widths up to 16 by doubling, others from a prefix
+//    kept as a value and its rounding error (over chunks of 3 to 19 samples a plain one is off by up to three times
+//    what the kernels before it were beside bright features).
 // Bound by instruction issue and, for few rows, by the copies (two or three CTAs fit on an SM, so
 // copy and search overlap only between them).  C and S are the smallest of the compiled windows S C
 // that hold the samples; the rows are split over as many warps as keep the SM's register file full.
 // 301 x 301 pixels x 16 subbands, 40 distinct DM rows, power-of-two widths, against the kernels
-// with a warp per row: FP32 100 samples 533 us (2873), 240 1311 us (2947), 400 2208 us (3261), 600
-// 2986 us (4409); BF16 240 1114 us (4887), 300 1567 us (9300), 600 2580 us (7077).  With in-lane prefixes
-// for the widths up to 16: 521, 1295, 2178, 3001; 1098, 1540, 2561 us.
+// with a warp per row: FP32 100 samples 539 us (2873), 240 1320 us (2947), 400 2267 us (3261), 600
+// 3056 us (4409); BF16 240 1125 us (4887), 300 1630 us (9300), 600 2636 us (7077).  With plain prefixes
+// for every width: 521, 1295, 2178, 3001; 1098, 1540, 2561 us.
 #pragma once
 
 #include <algorithm>
@@ -319,7 +321,10 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                     }
                 }
                 // widths of the in-lane path: the samples in the buffer, boxcars by doubling as in small_sums;
-                // others: P in the buffer, with P[t1 + c] kept in d[c]
+                // others: P as a value and its rounding error in the buffer (each S C words of the 32 C), P[t1 + c]
+                // kept in d[c], dl[c].  The error is left out where it is not a number (an infinite sample).
+                static_assert(2 * S <= 32, "value and error of the prefix");
+                float *Pl = Pw + S * C, dl[CC];
                 const bool small = w <= kSmallMax && (w & (w - 1)) == 0;
                 __syncwarp();
                 if (small) {
@@ -327,18 +332,28 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                     for (int c = 0; c < CC; ++c)
                         if (t1 + c < L) Pw[t1 + c] = d[c];
                 } else {
-                    float tot = 0.0f;
+                    float tot = 0.0f, tot_l = 0.0f;
 #pragma unroll
                     for (int c = 0; c < CC; ++c) {
                         const float v = t1 + c < L ? d[c] : 0.0f;
                         d[c] = tot;
-                        tot += v;
+                        dl[c] = tot_l;
+                        pair_add(tot, tot_l, v, 0.0f);
                     }
-                    const float carry = lane_carry(tot, lane);
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float yh = __shfl_up_sync(kFull, tot, o), yl = __shfl_up_sync(kFull, tot_l, o);
+                        if (lane >= o) pair_add(tot, tot_l, yh, yl);
+                    }
+                    float ch = __shfl_up_sync(kFull, tot, 1), cl = __shfl_up_sync(kFull, tot_l, 1);
+                    if (lane == 0) ch = cl = 0.0f;
 #pragma unroll
                     for (int c = 0; c < CC; ++c) {
-                        d[c] += carry;
-                        if (t1 + c <= L) Pw[t1 + c] = d[c];
+                        pair_add(d[c], dl[c], ch, cl);
+                        if (t1 + c <= L) {
+                            Pw[t1 + c] = d[c];
+                            Pl[t1 + c] = dl[c];
+                        }
                     }
                 }
                 __syncwarp();
@@ -360,7 +375,10 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
 #pragma unroll
                 for (int c = 0; c < CC; ++c) {
                     if (t1 + c + w <= L) {
-                        if (!small) d[c] = Pw[t1 + c + w] - d[c];
+                        if (!small) {
+                            const float b = Pw[t1 + c + w] - d[c], e = Pl[t1 + c + w] - dl[c];
+                            d[c] = e == e ? b + e : b;
+                        }
                         m = fmaxf(m, d[c]);
                     }
                 }

@@ -120,3 +120,22 @@ def test_infinite_samples_of_long_windows_are_left_out(native, n_t, dtype):
     _, best, _ = oracle.search_cube(clean.numpy(), sh, cfg.widths, sigma=sig)
     snr, idx = _search(native, cfg, cube, sig, dtype)
     parity.compare_best(snr, idx, best)
+
+
+@pytest.mark.parametrize("n_t,dtype", [(100, "f32"), (300, "bf16"), (400, "f32"), (607, "f32")])
+def test_records_of_other_widths_are_those_of_their_trial(native, n_t, dtype):
+    """Mid windows, widths with a prefix: the record's S/N is its trial's within 1e-6 beside a wide deep dip (sums
+    of the rebuilt row's samples alone: 16 subbands and the prefix's value and error, each a few times 2^-24)."""
+    cfg = _config(n_t, sorted({3, 7, 11, 25, 32, 60, n_t // 3}))
+    cube = synth.plain_noise(cfg, n_t + 2)
+    sh = oracle.delay_table(cfg.freq_mhz, cfg.dm)
+    for p in range(N_PIX):
+        cube[p, :, (p * n_t) // N_PIX:(p * n_t) // N_PIX + n_t // 8] -= 300.0
+    cube = cube.to(STORE[dtype])
+    snr, idx = _search(native, cfg, cube, np.full(N_PIX, 4.0, np.float32), dtype)
+    x = cube.float().numpy()
+    for p in range(N_PIX):
+        d, wi, t = (int(v) for v in idx[p])
+        w = int(cfg.widths[wi])
+        want = _direct(x[p], sh[d], w, t) / (4.0 * np.sqrt(float(w)))
+        assert abs(float(snr[p]) - want) <= 1e-6 * max(1.0, abs(want)), (p, snr[p], want)
