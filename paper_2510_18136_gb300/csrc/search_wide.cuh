@@ -84,6 +84,16 @@ __device__ __forceinline__ void team_sync(int team) {
     asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(THREADS) : "memory");
 }
 
+// box / (sigma sqrt(w)) with the divisor as a value and its rounding error and one correction of the quotient: the three
+// roundings of box inv, inv = 1 / (sigma sqrt(w)) in FP32, would be the largest error left in the record's S/N.
+__device__ __forceinline__ float wide_snr(float box, float sigma, int w, float inv) {
+    const float fw = static_cast<float>(w), r = sqrtf(fw);
+    const float den = sigma * r, lo = fmaf(sigma, r, -den) + sigma * (fmaf(-r, r, fw) / (2.0f * r));
+    const float q = box / den;
+    const float fix = (fmaf(-q, den, box) - q * lo) / den;
+    return fabsf(fix) <= 1e-6f * fabsf(q) ? q + fix : box * inv;   // (a divisor of 0 or infinity: no correction)
+}
+
 // Sums of the chunk's samples from each one to the chunk's end, as pairs (two chains, like prefix_pairs).
 template <int C>
 __device__ __forceinline__ void suffix_pairs(const float2 (&D)[C / 2], float2 (&S)[C / 2]) {
@@ -318,11 +328,12 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_wide(const __grid_c
                         else
                             return (cg.x + (next ? rest[A] : rest[A - 1])) + cg.y;
                     };
+                    const int first = v * kSeg;   // this segment's first sample: a width with no trial from it on is left out
                     // Width q C + r: trial c of the chunk ends in chunk + q, from c = C - r on in the one after.
                     // A trial that would leave the row reads what lies there, and adds -inf.
 #define NSFRB_WIDE_LARGE(J)                                                                                     \
     if constexpr ((1 << J) > kSmallMax) {                                                                       \
-        if (p.pow2_wi[J] >= 0) {                                                                                \
+        if (p.pow2_wi[J] >= 0 && first + (1 << J) <= L) {                                                       \
             constexpr int W = 1 << J, Q = W / C, R = W % C;                                                     \
             const float2 *x = reinterpret_cast<const float2 *>(Pt + min(t0 + W, (kChunks - 1) * C + R));        \
             float a[2] = {neg_inf(), neg_inf()};                                                                \
@@ -350,6 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_wide(const __grid_c
 #pragma unroll 1
                     for (int g = 0; g < p.n_gen; ++g) {
                         const int wi = p.gen_wi[g], w = p.widths[wi], q = w / C, r = w - q * C;
+                        if (first + w > L) continue;
                         const float *x = Pt + min(t0 + w, (kChunks - 1) * C + r), *own_p = Pw + lane * C;
                         const __half *own_lo = Low + lane * C;
                         auto link = [&](int g1) -> float {   // between, of chunk g1
@@ -516,7 +528,8 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_wide(const __grid_c
                         best = s_rm[g];
                         t = s_rt[g];
                     }
-                r = PixRec{best * s_inv[wi], s_info[u * kInfo + UI_FIRST_D], wi, t};
+                r = PixRec{wide_snr(best, p.sigma ? p.sigma[pix] : p.sigma_default, w, s_inv[wi]),
+                           s_info[u * kInfo + UI_FIRST_D], wi, t};
             }
             if (p.bad_pix && p.bad_pix[pix]) {
                 r = PixRec{neg_inf(), -1, -1, -1};
