@@ -126,7 +126,7 @@ def make_cube(native, synth, cfg, seed, device, dtype):
 # dram__bytes_write.sum of a 128x128 launch of search_kernel_team, 1263 MB, scaled by 90601 / 16384
 # pixels), valid for the kernel sources (the kernel and the row code it includes) with this sha256 prefix,
 # candidate records with the plan's default tile.
-NCU_TRAFFIC = {"sha256_16": "75c45ca75f241165", "bytes": (1.26e9 + 3.21e6) * 90601 / 16384,
+NCU_TRAFFIC = {"sha256_16": "4eb5b8d86b3487ac", "bytes": (1.26e9 + 2.90e6) * 90601 / 16384,
                "workload": (301, 301, 1200, 64, "f32", "candidates", 0)}
 
 

@@ -710,6 +710,15 @@ __device__ __forceinline__ void pair_add(float &h, float &l, float bh, float bl)
     h = s;
 }
 
+// A rebuilt record's S/N, box / (sigma sqrt(w)): box inv, inv = 1 / (sigma sqrt(w)) in FP32, and one correction of that
+// quotient by the divisor as a value and its rounding error.  Its four roundings would be the largest error left in it.
+__device__ __forceinline__ float record_snr(float box, float sigma, int w, float inv) {
+    const float fw = static_cast<float>(w), ri = inv * sigma, r = fw * ri;   // near 1 / sqrt(w) and sqrt(w)
+    const float den = sigma * r, lo = fmaf(sigma, r, -den) + sigma * (0.5f * ri * fmaf(-r, r, fw));
+    const float q = box * inv, fix = fmaf(-q, lo, fmaf(-q, den, box)) * inv;
+    return fabsf(fix) <= 1e-6f * fabsf(q) ? q + fix : q;   // (a divisor of 0 or infinity: no correction)
+}
+
 // Lane-strided P as pairs: Ps[m] = (P[64 m + lane], P[64 m + 32 + lane]).
 template <int C>
 __device__ __forceinline__ void load_ps(const float *Pw, int lane, float2 (&Ps)[C / 2]) {

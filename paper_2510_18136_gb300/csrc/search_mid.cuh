@@ -21,7 +21,7 @@
 //    a warp per pixel rebuilds the best row from all subbands, and takes the record's S/N and the
 //    earliest sample reaching it from that row: widths up to 16 by doubling, others from a prefix
 //    kept as a value and its rounding error (over chunks of 3 to 19 samples a plain one is off by up to three times
-//    what the kernels before it were beside bright features).
+//    what the kernels before it were beside bright features), the quotient corrected once.
 // Bound by instruction issue and, for few rows, by the copies (two or three CTAs fit on an SM, so
 // copy and search overlap only between them).  C and S are the smallest of the compiled windows S C
 // that hold the samples; the rows are split over as many warps as keep the SM's register file full.
@@ -383,12 +383,12 @@ __global__ void __launch_bounds__(C > 26 ? 192 : 256, 2) search_kernel_mid(const
                     }
                 }
                 m = warp_max(m);
-                r.snr = m * inv;
                 int at = INT_MAX;
 #pragma unroll
                 for (int c = CC - 1; c >= 0; --c)
-                    if (t1 + c + w <= L && d[c] * inv == r.snr) at = t1 + c;
+                    if (t1 + c + w <= L && d[c] * inv == m * inv) at = t1 + c;
                 at = warp_min(at);
+                r.snr = record_snr(m, p.sigma ? p.sigma[item_pixel(it0 + i)] : p.sigma_default, w, inv);
                 r.t_idx = at == INT_MAX ? -1 : at;
                 r.dm_idx = s_info[u * kInfo + UI_FIRST_D];
                 r.w_idx = wi;

@@ -17,7 +17,7 @@
 //    it is -inf or NaN and drops out of the maximum.
 //  * Only the best (row, width) is tracked.  At the end each pixel's best row is rebuilt from all
 //    subbands (the samples shared out over the warps), and the earliest sample reaching its
-//    maximum, with that maximum's S/N, goes to the record.
+//    maximum, with that maximum's S/N, goes to the record, the quotient corrected once.
 // Bound by instruction issue: per sample and row 1.5 operations per width, one for the prefix and
 // three per changed subband.  301 x 301 pixels x 16 subbands x 25 samples in FP32, 16 DM, 5 widths:
 // 106 us (1.4 TB/s), where the warp-per-row kernel with CTA barriers takes 3119 us; 16 binned samples,
@@ -305,9 +305,9 @@ search_kernel_short(const __grid_constant__ SearchParams p) {
                 auto box = [&](int t) { return fmaf(ca, a[t * sa], b[t * kShortPix]); };
                 float m = neg_inf();
                 for (int t = 0; t + w <= L; ++t) m = fmaxf(m, box(t));
-                r.snr = m * inv;
                 for (int t = L - w; t >= 0; --t)
-                    if (box(t) * inv == r.snr) r.t_idx = t;
+                    if (box(t) * inv == m * inv) r.t_idx = t;
+                r.snr = record_snr(m, p.sigma ? p.sigma[item_pixel(it0 + lane)] : p.sigma_default, w, inv);
                 r.dm_idx = s_info[bu * kInfo + UI_FIRST_D];
                 r.w_idx = bwi;
             }

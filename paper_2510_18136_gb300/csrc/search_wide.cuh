@@ -84,16 +84,6 @@ __device__ __forceinline__ void team_sync(int team) {
     asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(THREADS) : "memory");
 }
 
-// box / (sigma sqrt(w)) with the divisor as a value and its rounding error and one correction of the quotient: the three
-// roundings of box inv, inv = 1 / (sigma sqrt(w)) in FP32, would be the largest error left in the record's S/N.
-__device__ __forceinline__ float wide_snr(float box, float sigma, int w, float inv) {
-    const float fw = static_cast<float>(w), r = sqrtf(fw);
-    const float den = sigma * r, lo = fmaf(sigma, r, -den) + sigma * (fmaf(-r, r, fw) / (2.0f * r));
-    const float q = box / den;
-    const float fix = (fmaf(-q, den, box) - q * lo) / den;
-    return fabsf(fix) <= 1e-6f * fabsf(q) ? q + fix : box * inv;   // (a divisor of 0 or infinity: no correction)
-}
-
 // Sums of the chunk's samples from each one to the chunk's end, as pairs (two chains, like prefix_pairs).
 template <int C>
 __device__ __forceinline__ void suffix_pairs(const float2 (&D)[C / 2], float2 (&S)[C / 2]) {
@@ -528,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1) search_kernel_wide(const __grid_c
                         best = s_rm[g];
                         t = s_rt[g];
                     }
-                r = PixRec{wide_snr(best, p.sigma ? p.sigma[pix] : p.sigma_default, w, s_inv[wi]),
+                r = PixRec{record_snr(best, p.sigma ? p.sigma[pix] : p.sigma_default, w, s_inv[wi]),
                            s_info[u * kInfo + UI_FIRST_D], wi, t};
             }
             if (p.bad_pix && p.bad_pix[pix]) {

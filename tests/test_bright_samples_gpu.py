@@ -139,3 +139,21 @@ def test_records_of_other_widths_are_those_of_their_trial(native, n_t, dtype):
         w = int(cfg.widths[wi])
         want = _direct(x[p], sh[d], w, t) / (4.0 * np.sqrt(float(w)))
         assert abs(float(snr[p]) - want) <= 1e-6 * max(1.0, abs(want)), (p, snr[p], want)
+
+
+@pytest.mark.parametrize("n_t,dtype", [(1, "f32"), (25, "f32"), (62, "bf16"), (64, "f16"), (65, "f32"), (300, "bf16"),
+                                       (607, "f32"), (1248, "f32"), (2400, "bf16"), (4096, "bf16")])
+def test_record_is_its_boxcar_divided_once(native, n_t, dtype):
+    """Short, mid and long windows: of integer samples every boxcar is exact, and what is left is the quotient
+    box / (sigma sqrt(w)), rounded once: half a unit in the last place, 2^-24 of it at most (and its square)."""
+    cfg = _config(n_t, sorted({w for w in (1, 2, 4, 7, 16, 50, 200, n_t) if w <= n_t}))
+    rng = np.random.default_rng(n_t)
+    x = rng.integers(-100, 101, (N_PIX, 16, n_t)).astype(np.float32)     # sums below 2^24
+    sig = rng.uniform(0.7, 300.0, N_PIX).astype(np.float32)
+    sh = oracle.delay_table(cfg.freq_mhz, cfg.dm)
+    snr, idx = _search(native, cfg, torch.from_numpy(x).to(STORE[dtype]), sig, dtype)
+    for p in range(N_PIX):
+        d, wi, t = (int(v) for v in idx[p])
+        w = int(cfg.widths[wi])
+        want = _direct(x[p], sh[d], w, t) / (float(sig[p]) * np.sqrt(float(w)))
+        assert abs(float(snr[p]) - want) <= 1.01 * 2.0 ** -24 * abs(want), (p, snr[p], want)
