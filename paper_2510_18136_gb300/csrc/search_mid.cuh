@@ -26,8 +26,8 @@
 // copy and search overlap only between them).  C and S are the smallest of the compiled windows S C
 // that hold the samples; the rows are split over as many warps as keep the SM's register file full.
 // 301 x 301 pixels x 16 subbands, 40 distinct DM rows, power-of-two widths, against the kernels
-// with a warp per row: FP32 100 samples 539 us (2873), 240 1320 us (2947), 400 2267 us (3261), 600
-// 3056 us (4409); BF16 240 1125 us (4887), 300 1630 us (9300), 600 2636 us (7077).  With plain prefixes
+// with a warp per row: FP32 100 samples 539 us (2873), 240 1324 us (2947), 400 2270 us (3261), 600
+// 3059 us (4409); BF16 240 1127 us (4887), 300 1630 us (9300), 600 2638 us (7077).  With plain prefixes
 // for every width: 521, 1295, 2178, 3001; 1098, 1540, 2561 us.
 #pragma once
 

@@ -21,7 +21,7 @@
 //    fit (16-bit rows, shorter FP32 windows), else it starts when the rows have been read for the last time.
 // Bound by the reads of Lp (66 % of L1's throughput at 2048 FP32 samples, issue 50 %).  9696 pixels x 16
 // subbands, 40 distinct DM rows, 12 widths, against the long-window kernel: 1250 samples FP32
-// 1.37 ms (7.44), 2048 1.73 ms (11.9), BF16 1.73 ms (16.4), 3000 2.48 ms (27.3), 4096 3.19 ms (38.5).  With
+// 1.35 ms (7.44), 2048 1.70 ms (11.9), BF16 1.70 ms (16.4), 3000 2.45 ms (27.3), 4096 3.15 ms (38.5).  With
 // one FP32 prefix per segment and differences of it the same searches take 1.22, 1.54, 1.52, 2.10
 // and 2.81 ms, but beside a dip of -300 a sample over 256 of 2048 samples the relative error of the S/N
 // reaches 6e-4 (here 1.4e-7, the long-window kernel 2.4e-6), and a sample that is not a number left
